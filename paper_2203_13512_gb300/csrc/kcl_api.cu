@@ -379,6 +379,7 @@ kcl_status run_call(kcl_graph *g, uint32_t k, kcl_ordering ord, const kcl_ring *
         size_t arena = ord == KCL_ORDER_DEGREE
                            ? sdegree_arena_words(k, g->num_sms, fe.max_outdeg)
                            : bitcol_arena_words(k, g->num_sms, fe.max_outdeg);
+        if (k <= 6) arena = std::max(arena, sub_arena_words(g->num_sms, fe.max_outdeg, listing));
         KCL_TRY(ensure_arena(g, arena));
         int l = ord == KCL_ORDER_DEGREE
                     ? launch_sdegree(g, k, w, fe.class_begin, fe.n_classes, la, g->stream)

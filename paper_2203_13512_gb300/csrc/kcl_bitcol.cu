@@ -1116,6 +1116,11 @@ int launch_bitcol(const kcl_graph *g, uint32_t k, Workspace &w, const uint32_t *
         if (cc.cta) class_layout(c, la.max_outdeg, &Wl, &Dl);
         const size_t smem = cc.cta ? class_smem(c, k, Wl, Dl) : class_smem(c, k);
         class_mark(la, c, 0, s);
+        if (sub_handles(g, k, c, KCL_ORDER_COLOR)) {
+            launches += launch_sub(g, k, w, c, begin, end, q, la, em.dfs_warps, s);
+            class_mark(la, c, 1, s);
+            continue;
+        }
         if (!cc.cta && la.listing) {
             // listing: every clique is hashed one by one, so a root's cost grows
             // with its clique count; a CTA of 4 warps shares each root's

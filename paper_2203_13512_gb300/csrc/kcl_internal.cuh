@@ -564,6 +564,13 @@ int launch_bitcol_colours(const Workspace &w, uint32_t u, uint32_t d, uint32_t *
 int launch_bitcol(const kcl_graph *g, uint32_t k, Workspace &w, const uint32_t *class_begin,
                   int n_classes, const ListArgs &la, cudaStream_t s);
 
+// kcl_sub.cu: id-ordered subproblems (k <= 6, d+ <= 1024), both orderings.
+// sub_handles: whether class c of a call (k: the largest of a batch) runs there.
+bool sub_handles(const kcl_graph *g, uint32_t k, int c, kcl_ordering ord);
+size_t sub_arena_words(int num_sms, uint32_t max_outdeg, bool listing);
+int launch_sub(const kcl_graph *g, uint32_t k, Workspace &w, int c, uint32_t begin, uint32_t end, unsigned *queue,
+               const ListArgs &la, uint32_t dfs_warps, cudaStream_t s);
+
 // kcl_sdegree.cu
 int sdegree_classes(uint32_t *limits, int max);
 size_t sdegree_arena_words(uint32_t k, int num_sms, uint32_t max_outdeg);

@@ -1598,6 +1598,11 @@ int launch_sdegree(const kcl_graph *g, uint32_t k, Workspace &w, const uint32_t 
         em.split = cta_form ? g->tuning.sdegree_split[c] : 0u;
         if (em.split) cudaMemsetAsync(w.slots, 0xFF, kMaxSplitSlots * sizeof(unsigned long long), s);
         class_mark(la, c, 0, s);
+        if (sub_handles(g, k, c, KCL_ORDER_DEGREE)) {
+            launches += launch_sub(g, k, w, c, begin, end, q, la, dw, s);
+            class_mark(la, c, 1, s);
+            continue;
+        }
         if (c < kWarpClasses) {
             // listing hashes every clique: a root's cost grows with its clique
             // count, so listing shares each root's children over a CTA of 4 warps
