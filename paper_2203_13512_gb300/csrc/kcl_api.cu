@@ -225,21 +225,10 @@ kcl_status status_from_device(uint32_t st) {
     return KCL_OK;
 }
 
-// Degeneracy peel in one cooperative launch (false: not launchable here, the
+// Degeneracy peel on co-resident blocks (false: not launchable here, the
 // caller falls back to one launch per round).
-bool run_peel_coop(kcl_graph *g, StageTimer &T) {
-    Workspace &w = g->ws;
-    cudaStream_t s = g->stream;
-    if (cudaMemsetAsync(w.peel, 0, sizeof(PeelCtl), s) != cudaSuccess ||
-        cudaMemsetAsync(w.peel->minv, 0xFF, sizeof(w.peel->minv), s) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return false;
-    }
-    // the remaining-vertex lists (n words each) and the big-row lists (n / 2
-    // each) use the root-histogram scratch (3n + 1024 words), which is free
-    // until the roots are sorted after the peel
-    const size_t n = g->n;
-    int l = launch_peel_coop(g, w, w.peel, w.hist, w.hist + n, w.hist + 2 * n, w.hist + 2 * n + n / 2 + 1, s);
+bool run_peel(kcl_graph *g, StageTimer &T) {
+    const int l = launch_peel(g, g->ws, g->stream);
     if (l < 0) {
         (void)cudaGetLastError();
         return false;
@@ -287,7 +276,7 @@ kcl_status run_front(kcl_graph *g, uint32_t k, kcl_ordering ord, const kcl_ring 
     T.begin(2);
     if (ord == KCL_ORDER_DEGREE) {
         T.add(2, launch_degree_key(g, w, s));
-    } else if (run_peel_coop(g, T)) {
+    } else if (run_peel(g, T)) {
         uint32_t err = 0;
         KCL_CK(cudaMemcpyAsync(&err, &w.peel->error, sizeof(err), cudaMemcpyDeviceToHost, s));
         KCL_CK(cudaStreamSynchronize(s));

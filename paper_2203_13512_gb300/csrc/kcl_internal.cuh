@@ -42,16 +42,31 @@ struct DevResult {
     unsigned long long deadline_ns;  // %globaltimer value after which listing stops (0: none)
 };
 
-// Control block of the single-launch degeneracy peel: grid barrier state,
-// the number of vertices to peel, frontier sizes (rotating over three rounds),
-// remaining-list sizes and minimum degrees (alternating over threshold
-// levels).  All zero at launch except minv, all ones.
+// Counters of the degeneracy peel's rounds (all zero at launch): frontier
+// sizes and big-row counts rotate over three rounds; the minimum degree of a
+// threshold pass (kept as 0x80000000 - degree) and the vertices it selects
+// rotate over four passes.
+struct PeelCounters {
+    unsigned fcnt[3], bcnt[3], top[4], sel[4], near;
+};
+
+// Where the rounds stand: vertices removed before this round, this round's
+// number and size, the threshold t, the bound B of the near list, all vertices.
+struct PeelState {
+    unsigned done, nin, round;
+    int t, B;
+    unsigned total;
+};
+
+// Control block of the peel: grid barrier state, the grid's counters, the
+// state it hands to the cluster and the long rows of a round.  All zero at
+// launch.
+constexpr unsigned kPeelBig = 256;
 struct PeelCtl {
-    unsigned bar_count, bar_gen, error, remaining;
-    unsigned fcnt[3];   // frontier sizes (vertices up to the big-degree threshold)
-    unsigned rcnt[2];
-    unsigned minv[2];
-    unsigned bcnt[3];   // big-vertex frontier sizes (rotating like fcnt)
+    unsigned bar_count, bar_gen, error, total;
+    PeelCounters cnt;
+    PeelState st;
+    unsigned big[3][kPeelBig];
 };
 
 // One graph of a batch: its device CSR and its place in the disjoint union.
@@ -515,13 +530,9 @@ int launch_peel_select_all(const kcl_graph *g, Workspace &w, uint32_t t, uint32_
 int launch_peel_update(const kcl_graph *g, Workspace &w, const uint32_t *fin, uint32_t nin,
                        uint32_t t, uint32_t round, uint32_t *fout, cudaStream_t s);
 int launch_peel_min(const kcl_graph *g, Workspace &w, cudaStream_t s);
-// Whole degeneracy peel in one cooperative launch; -1 if it cannot launch.
-// rl0/rl1: two n-entry arrays for the compacted remaining-vertex lists (or
-// both null: every threshold rise scans all n vertices); bl0/bl1: two
-// n/2-entry arrays for the frontier's big-degree vertices, whose rows the
-// whole grid walks together (or null: every frontier vertex takes one warp).
-int launch_peel_coop(const kcl_graph *g, Workspace &w, PeelCtl *ctl, uint32_t *rl0, uint32_t *rl1,
-                     uint32_t *bl0, uint32_t *bl1, cudaStream_t s);
+// Whole degeneracy peel in one or two launches of co-resident blocks (clears
+// w.peel first); -1 if it cannot launch.
+int launch_peel(const kcl_graph *g, Workspace &w, cudaStream_t s);
 int launch_orient(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s);
 int launch_roots(const kcl_graph *g, uint32_t k, Workspace &w, uint32_t max_outdeg,
                  uint32_t *class_begin, const uint32_t *class_limits, int n_classes,

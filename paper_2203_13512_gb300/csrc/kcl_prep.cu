@@ -4,6 +4,7 @@
 // the out-neighbour CSR of the DAG, plus the root list the listing kernels
 // consume.  Every pass here streams the CSR once: these kernels are bound by
 // HBM bandwidth, so they use warp-per-vertex row scans with coalesced loads.
+#include <algorithm>
 #include <mutex>
 
 #include "kcl_internal.cuh"
@@ -365,24 +366,35 @@ __global__ void k_peel_update(const uint64_t *__restrict__ rp, const uint32_t *_
     }
 }
 
-// The same peel in one cooperative launch (every block resident): rounds are
-// separated by a grid barrier instead of a kernel boundary and a host round
-// trip.  Every block follows the same control flow, derived from counters
-// read after a barrier:
-//   a round with a non-empty frontier (a cascade) processes it and ends with
-//     one barrier; frontier counters rotate over three rounds (round r reads
-//     fcnt[r % 3], appends to fcnt[(r+1) % 3] and clears fcnt[(r+2) % 3],
-//     which every block read two barriers earlier);
-//   a round with an empty frontier raises t: a pass over the remaining
-//     vertices finds their minimum degree (barrier), a second pass selects
-//     those at or below t into the frontier and, when rl0/rl1 are given,
-//     compacts the vertices still remaining into the other list (barrier),
-//     so later passes touch only what is left.
-// Arrays written during the launch are read with ld.global.cg (L2) so no
-// stale L1 line is used.  Every barrier wait is bounded: past kSpinLimit
-// polls the block records an error, all blocks leave, and the host reports
-// KCL_ETIMEOUT.
+// The same peel in one launch of co-resident blocks: rounds are separated by
+// a barrier instead of a kernel boundary and a host round trip.  A graph has
+// hundreds of rounds with little work each (660 on R-MAT 20, most of them one
+// threshold step with a few vertices), so a round's chain of dependent memory
+// accesses and barriers is what bounds the peel:
+//   - a vertex is gone once its degree is at or below t, so relaxing an edge
+//     is one atomic on the neighbour's degree, with no look at its key or alive
+//     flag (vertices that are not alive hold a degree far below zero); the
+//     thread that sees t + 1 -> t, and only that one, puts it in the next round;
+//   - a threshold step looks only at the near list, the vertices whose degree
+//     lies in (t, B]; a relaxation that sees B + 1 -> B adds to it, and a pass
+//     over all vertices starts a new one every kNear thresholds;
+//   - a round with few vertices spreads each row over several warps;
+//   - the whole grid runs the wide first rounds (grid barrier, about 2 us), one
+//     cluster of at most 16 CTAs the long tail, with its hardware barrier and the
+//     counters in the first CTA's shared memory.
+// On the 1M-vertex R-MAT graph (678 rounds) this took the peel from 17.5 to 6.3
+// ms, about 7 us a round in the cluster, 3.4 us on 65k vertices.
+// Every thread follows the same control flow, derived from counters read after
+// a barrier; frontier and big-row counters rotate over three rounds (round r
+// reads slot r % 3, appends to (r + 1) % 3 and clears (r + 2) % 3, which
+// everybody read two barriers earlier).  Arrays written during the launch are
+// read with ld.global.cg (L2) so no stale L1 line is used.  Every grid-barrier
+// wait is bounded: past kSpinLimit polls the block records an error, all blocks
+// leave, and the host reports KCL_ETIMEOUT.
 constexpr unsigned long long kSpinLimit = 1ull << 25;
+constexpr int kNear = 32;                 // thresholds a near list covers
+constexpr uint32_t kBigRow = 4096;        // longer rows are walked by all warps
+constexpr int kGone = -(1 << 30);         // degree of a vertex that is not alive
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
     unsigned v;
@@ -423,148 +435,263 @@ __device__ bool grid_barrier(PeelCtl *c, unsigned nblocks) {
     return ok_s != 0;
 }
 
-// A frontier vertex whose row is longer than `big` goes to a separate list
-// (bl0/bl1 by round parity) and its row is walked by every thread of the grid
-// instead of one warp, so a hub does not stretch its round.
-__global__ void __launch_bounds__(1024) k_peel_coop(uint32_t n, const uint64_t *__restrict__ rp,
-                                                    const uint32_t *__restrict__ col,
-                                                    const uint8_t *__restrict__ alive,
-                                                    const uint32_t *__restrict__ cdeg, uint32_t *pdeg,
-                                                    uint32_t *key, uint32_t *fa, uint32_t *fb,
-                                                    uint32_t *rl0, uint32_t *rl1, uint32_t *bl0,
-                                                    uint32_t *bl1, uint64_t big, PeelCtl *c) {
-    const unsigned nblocks = gridDim.x;
-    const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t nth = gridDim.x * blockDim.x;
+struct PeelArgs {
+    uint32_t n;
+    const uint64_t *rp;
+    const uint32_t *col;
+    const uint8_t *alive;
+    const uint32_t *cdeg;
+    int *deg;          // degrees during the peel
+    uint32_t *key;     // round a vertex leaves in
+    uint32_t *order;   // vertices in the order they leave: round r's frontier is a range
+    uint32_t *near;    // near list
+    PeelCtl *ctl;
+    uint32_t handover; // grid: leave the rest to the cluster at this many vertices
+};
+
+struct GridSync {
+    PeelCtl *ctl;
+    unsigned nblocks;
+    __device__ __forceinline__ bool operator()() const { return grid_barrier(ctl, nblocks); }
+};
+struct ClusterSync {
+    __device__ __forceinline__ bool operator()() const {
+        asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
+        return true;
+    }
+};
+
+// One warp's lanes append to a list: the position of this lane's entry.
+__device__ __forceinline__ uint32_t warp_append(unsigned m, unsigned *count) {
     const unsigned lane = lane_id();
-    volatile PeelCtl *vc = c;
-    const bool lists = rl0 != nullptr;
-    {
-        uint32_t cnt = 0;
-        for (uint32_t v0 = tid - lane; v0 < n; v0 += nth) {  // warp-uniform trip count
-            const uint32_t v = v0 + lane;
-            bool a = false;
-            if (v < n) {
-                pdeg[v] = cdeg[v];
-                key[v] = 0xFFFFFFFFu;
-                a = alive[v] != 0;
-            }
-            cnt += a ? 1 : 0;
-            if (lists) {  // the first remaining list: every alive vertex
-                const unsigned m = __ballot_sync(0xffffffffu, a);
-                unsigned base = 0;
-                if (lane == 0 && m) base = atomicAdd(&c->rcnt[0], (unsigned)__popc(m));
-                base = __shfl_sync(0xffffffffu, base, 0);
-                if (a) rl0[base + __popc(m & ((1u << lane) - 1u))] = v;
+    uint32_t base = 0;
+    if (lane == 0) base = atomicAdd(count, (unsigned)__popc(m));
+    return __shfl_sync(0xffffffffu, base, 0) + __popc(m & ((1u << lane) - 1u));
+}
+
+// Degrees, keys and the number of vertices to peel.
+__device__ void peel_setup(const PeelArgs &a, uint32_t tid, uint32_t nth, unsigned *total) {
+    uint32_t cnt = 0;
+    for (uint32_t v0 = tid - lane_id(); v0 < a.n; v0 += nth) {  // warp-uniform trip count
+        const uint32_t v = v0 + lane_id();
+        if (v < a.n) {
+            const bool on = a.alive[v] != 0;
+            a.deg[v] = on ? (int)a.cdeg[v] : kGone;
+            a.key[v] = 0xFFFFFFFFu;
+            cnt += on ? 1 : 0;
+        }
+    }
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane_id() == 0 && cnt) atomicAdd(total, cnt);
+}
+
+// Lowers the degrees of up to four neighbours a lane (n of them valid, stride
+// `step` from x) and appends those that reach t or B.
+__device__ __forceinline__ void peel_relax(const PeelArgs &a, PeelCounters *c, unsigned *next, uint32_t next0,
+                                           uint64_t x, uint64_t e, uint64_t step, int t, int B, uint32_t round) {
+    uint32_t w[4];
+    int old[4];
+#pragma unroll
+    for (int z = 0; z < 4; z++) w[z] = x + z * step < e ? a.col[x + z * step] : 0xFFFFFFFFu;
+#pragma unroll
+    for (int z = 0; z < 4; z++) old[z] = w[z] != 0xFFFFFFFFu ? atomicSub(&a.deg[w[z]], 1) : kGone;
+#pragma unroll
+    for (int z = 0; z < 4; z++) {
+        const bool join = old[z] == t + 1;
+        const unsigned m = __ballot_sync(0xffffffffu, join);
+        if (m) {
+            const uint32_t at = warp_append(m, next);
+            if (join) {
+                a.order[next0 + at] = w[z];
+                a.key[w[z]] = round + 1;
             }
         }
-        cnt = __reduce_add_sync(0xffffffffu, cnt);
-        if (lane == 0 && cnt) atomicAdd(&c->remaining, cnt);
+        const bool close = old[z] == B + 1 && B > t;
+        const unsigned mc = __ballot_sync(0xffffffffu, close);
+        if (mc) {
+            const uint32_t at = warp_append(mc, &c->near);
+            if (close) a.near[at] = w[z];
+        }
     }
-    if (!grid_barrier(c, nblocks)) return;
-    uint32_t remaining = vc->remaining;
-    uint32_t round = 0, t = 0, level = 0;
-    while (remaining > 0) {
-        const uint32_t fi = round % 3u;
-        uint32_t *fin = (round & 1u) ? fb : fa;
-        uint32_t *fout = (round & 1u) ? fa : fb;
-        uint32_t *bin = (round & 1u) ? bl1 : bl0;
-        uint32_t *bout = (round & 1u) ? bl0 : bl1;
-        uint32_t nin = vc->fcnt[fi];
-        uint32_t nbig = vc->bcnt[fi];
-        if (nin + nbig == 0) {
-            // t rises to the minimum remaining degree
-            const uint32_t lp = level & 1u;
-            const uint32_t *rl = lp ? rl1 : rl0;
-            uint32_t *rl_next = lp ? rl0 : rl1;
-            const uint32_t nr = lists ? vc->rcnt[lp] : n;
-            if (tid == 0 && lists) c->rcnt[lp ^ 1u] = 0;  // read at the previous level
-            uint32_t mn = 0xFFFFFFFFu;
-            for (uint32_t i = tid; i < nr; i += nth) {
-                const uint32_t v = lists ? __ldcg(&rl[i]) : i;
-                if ((lists || alive[v]) && __ldcg(&key[v]) == 0xFFFFFFFFu) {
-                    const uint32_t d = __ldcg(&pdeg[v]);
-                    mn = d < mn ? d : mn;
-                }
-            }
-            mn = __reduce_min_sync(0xffffffffu, mn);
-            if (lane == 0 && mn != 0xFFFFFFFFu) atomicMin(&c->minv[lp], mn);
-            if (!grid_barrier(c, nblocks)) return;
-            const uint32_t mv = vc->minv[lp];
-            if (mv > t) t = mv;
-            if (tid == 0) c->minv[lp ^ 1u] = 0xFFFFFFFFu;  // read at the previous level
-            // select the frontier; compact the rest into the other list
-            for (uint32_t i0 = tid - lane; i0 < nr; i0 += nth) {
-                const uint32_t i = i0 + lane;
-                bool sel = false, keep = false, sbig = false;
-                uint32_t v = 0;
-                if (i < nr) {
-                    v = lists ? __ldcg(&rl[i]) : i;
-                    if ((lists || alive[v]) && __ldcg(&key[v]) == 0xFFFFFFFFu) {
-                        sel = __ldcg(&pdeg[v]) <= t;
-                        keep = !sel;
-                        sbig = sel && bl0 && rp[v + 1] - rp[v] > big;
-                        sel = sel && !sbig;
+}
+
+// The rounds from state `st` on; every thread of the group calls it with the
+// same state.  Returns when at most `stop` vertices remain (0: all peeled),
+// with the state to resume from; false when a barrier gave up.
+template <typename Sync>
+__device__ bool peel_rounds(const PeelArgs &a, PeelCounters *c, PeelState &st, uint32_t stop, uint32_t tid,
+                            uint32_t nth, const Sync &sync) {
+    volatile PeelCounters *vc = c;
+    const unsigned lane = lane_id();
+    const uint32_t gw = tid >> 5, W = nth >> 5;
+    uint32_t q = 0;  // threshold passes so far (minimum slots rotate over four)
+    while (st.done < st.total && st.total - st.done > stop) {
+        const uint32_t fi = st.round % 3u;
+        if (st.nin == 0) {
+            // every remaining degree is above t: raise t to their minimum
+            for (;;) {
+                const uint32_t slot = q++ & 3u;
+                if (tid == 0) c->top[(slot + 2) & 3u] = c->sel[(slot + 2) & 3u] = 0;
+                const bool fresh = st.t + 1 > st.B;  // no near list for t + 1: start one
+                uint32_t best = 0;  // of 0x80000000 - degree: the maximum marks the minimum degree
+                if (fresh) {
+                    if (tid == 0) c->near = 0;
+                    if (!sync()) return false;
+                    const int B = st.t + kNear;
+                    for (uint32_t v0 = tid - lane; v0 < a.n; v0 += nth) {
+                        const uint32_t v = v0 + lane;
+                        const int d = v < a.n ? __ldcg(&a.deg[v]) : kGone;
+                        const bool rest = d > st.t, in = rest && d <= B;
+                        if (rest) best = max(best, 0x80000000u - (uint32_t)d);
+                        const unsigned m = __ballot_sync(0xffffffffu, in);
+                        if (m) {
+                            const uint32_t at = warp_append(m, &c->near);
+                            if (in) a.near[at] = v;
+                        }
+                    }
+                } else {
+                    const uint32_t nn = vc->near;
+                    for (uint32_t i0 = tid - lane; i0 < nn; i0 += nth) {
+                        const uint32_t i = i0 + lane;
+                        uint32_t v = 0;
+                        int d = kGone;
+                        if (i < nn) {
+                            v = __ldcg(&a.near[i]);
+                            d = __ldcg(&a.deg[v]);
+                        }
+                        if (d > st.t) best = max(best, 0x80000000u - (uint32_t)d);
+                        const bool sel = d == st.t + 1;
+                        const unsigned m = __ballot_sync(0xffffffffu, sel);
+                        if (m) {
+                            const uint32_t at = warp_append(m, &c->sel[slot]);
+                            if (sel) {
+                                a.order[st.done + at] = v;
+                                a.key[v] = st.round;
+                            }
+                        }
                     }
                 }
-                const unsigned ms = __ballot_sync(0xffffffffu, sel);
-                unsigned bs = 0;
-                if (lane == 0 && ms) bs = atomicAdd(&c->fcnt[fi], (unsigned)__popc(ms));
-                bs = __shfl_sync(0xffffffffu, bs, 0);
-                if (sel) {
-                    key[v] = round;
-                    fin[bs + __popc(ms & ((1u << lane) - 1u))] = v;
+                best = __reduce_max_sync(0xffffffffu, best);
+                if (lane == 0 && best) atomicMax(&c->top[slot], best);
+                if (!sync()) return false;
+                const uint32_t top = vc->top[slot];
+                const int mn = top ? (int)(0x80000000u - top) : 0;
+                if (fresh) {
+                    if (!top) {  // cannot happen while vertices remain
+                        if (tid == 0) atomicExch(&a.ctl->error, 2u);
+                        return false;
+                    }
+                    const int B = st.t + kNear;
+                    st.t = mn - 1;
+                    st.B = mn <= B ? B : st.t;  // nothing up to B: start over from the minimum
+                    continue;
                 }
-                if (sbig) {  // rare: one atomic each
-                    key[v] = round;
-                    bin[atomicAdd(&c->bcnt[fi], 1u)] = v;
+                st.nin = vc->sel[slot];
+                if (st.nin) {
+                    st.t++;
+                    break;
                 }
-                if (lists) {
-                    const unsigned mk = __ballot_sync(0xffffffffu, keep);
-                    unsigned bk = 0;
-                    if (lane == 0 && mk) bk = atomicAdd(&c->rcnt[lp ^ 1u], (unsigned)__popc(mk));
-                    bk = __shfl_sync(0xffffffffu, bk, 0);
-                    if (keep) rl_next[bk + __popc(mk & ((1u << lane) - 1u))] = v;
-                }
-            }
-            level++;
-            if (!grid_barrier(c, nblocks)) return;
-            nin = vc->fcnt[fi];
-            nbig = vc->bcnt[fi];
-            if (nin + nbig == 0) {  // cannot happen while vertices remain
-                if (tid == 0) atomicExch(&c->error, 2u);
-                return;
+                if (top) st.t = mn - 1;  // the near list's minimum is higher
+                else st.B = st.t;        // the near list is used up
             }
         }
-        if (tid == 0) {  // every block read these two barriers ago
-            c->fcnt[(round + 2u) % 3u] = 0;
-            c->bcnt[(round + 2u) % 3u] = 0;
+        if (tid == 0) {
+            c->fcnt[(st.round + 2u) % 3u] = 0;
+            c->bcnt[(st.round + 1u) % 3u] = 0;
         }
-        // remove this round's vertices: lower the degrees of their remaining
-        // neighbours; a neighbour reaching <= t joins the next round
-        uint32_t *fnext_cnt = &c->fcnt[(round + 1u) % 3u];
-        uint32_t *bnext_cnt = &c->bcnt[(round + 1u) % 3u];
-        auto relax = [&](uint32_t w) {
-            if (!alive[w] || __ldcg(&key[w]) != 0xFFFFFFFFu) return;
-            const uint32_t nd = atomicSub(&pdeg[w], 1u) - 1u;
-            if (nd <= t && atomicCAS(&key[w], 0xFFFFFFFFu, round + 1) == 0xFFFFFFFFu) {
-                if (bl0 && rp[w + 1] - rp[w] > big) bout[atomicAdd(bnext_cnt, 1u)] = w;
-                else fout[atomicAdd(fnext_cnt, 1u)] = w;
+        // remove this round's vertices
+        unsigned *next = &c->fcnt[(st.round + 1u) % 3u];
+        unsigned *bcnt = &c->bcnt[fi];
+        uint32_t *big = a.ctl->big[fi];
+        const uint32_t next0 = st.done + st.nin;
+        uint32_t ls = 0;  // log2 of the warps per row
+        while ((st.nin << (ls + 1)) <= W) ls++;
+        for (uint32_t unit = gw; unit < st.nin << ls; unit += W) {
+            const uint32_t v = __ldcg(&a.order[st.done + (unit >> ls)]);
+            const uint64_t b = a.rp[v], e = a.rp[v + 1];
+            if (ls == 0 && e - b > kBigRow) {
+                uint32_t at = 0;
+                if (lane == 0) at = atomicAdd(bcnt, 1u);
+                at = __shfl_sync(0xffffffffu, at, 0);
+                if (at < kPeelBig) {
+                    if (lane == 0) big[at] = v;
+                    continue;
+                }
             }
-        };
-        for (uint32_t b = 0; b < nbig; b++) {  // big rows: the whole grid, one edge per thread
-            const uint32_t v = __ldcg(&bin[b]);
-            for (uint64_t e = rp[v] + tid; e < rp[v + 1]; e += nth) relax(col[e]);
+            const uint64_t step = 32ull << ls;
+            for (uint64_t x = b + 32 * (unit & ((1u << ls) - 1u)); x < e; x += 4 * step)
+                peel_relax(a, c, next, next0, x + lane, e, step, st.t, st.B, st.round);
         }
-        for (uint32_t i = tid >> 5; i < nin; i += nth >> 5) {
-            const uint32_t v = __ldcg(&fin[i]);
-            for (uint64_t e = rp[v] + lane; e < rp[v + 1]; e += 32) relax(col[e]);
+        if (!sync()) return false;
+        const uint32_t nb = min(vc->bcnt[fi], (unsigned)kPeelBig);
+        if (nb) {
+            for (uint32_t i = 0; i < nb; i++) {
+                const uint32_t v = __ldcg(&big[i]);
+                const uint64_t b = a.rp[v], e = a.rp[v + 1];
+                for (uint64_t x = b + (uint64_t)gw * 32; x < e; x += 4ull * nth)
+                    peel_relax(a, c, next, next0, x + lane, e, nth, st.t, st.B, st.round);
+            }
+            if (!sync()) return false;
         }
-        const uint32_t gone = nin + nbig;
-        remaining -= gone < remaining ? gone : remaining;
-        round++;
-        if (!grid_barrier(c, nblocks)) return;
+        st.done = next0;
+        st.round++;
+        st.nin = vc->fcnt[st.round % 3u];
     }
+    return true;
+}
+
+// The wide rounds, all SMs.
+__global__ void __launch_bounds__(1024) k_peel_grid(const PeelArgs a) {
+    PeelCounters *c = &a.ctl->cnt;
+    const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+    const GridSync sync{a.ctl, gridDim.x};
+    peel_setup(a, tid, nth, &a.ctl->total);
+    if (!sync()) return;
+    PeelState st{0, 0, 0, -1, -1, *(volatile unsigned *)&a.ctl->total};
+    if (!peel_rounds(a, c, st, a.handover, tid, nth, sync)) return;
+    if (tid == 0) a.ctl->st = st;
+}
+
+// The rest (or, for small graphs, all of it: resume = 0) in one cluster.
+__global__ void __launch_bounds__(1024) k_peel_cluster(const PeelArgs a, int resume) {
+    __shared__ PeelCounters own;
+    __shared__ unsigned total;
+    uint32_t rank, csize;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(csize));
+    const uint32_t tid = rank * blockDim.x + threadIdx.x, nth = csize * blockDim.x;
+    const ClusterSync sync;
+    if (resume && a.ctl->error) return;  // the grid's rounds gave up: every thread leaves
+    if (threadIdx.x == 0) {
+        own = PeelCounters{};
+        total = 0;
+        if (resume) {
+            own = a.ctl->cnt;
+            for (int i = 0; i < 4; i++) own.top[i] = own.sel[i] = 0;  // threshold passes start over
+        }
+    }
+    // the first CTA's counters, by their address in the cluster's shared memory
+    PeelCounters *c;
+    unsigned *tot;
+    {
+        uint64_t p = reinterpret_cast<uint64_t>(&own), r;
+        asm("mapa.u64 %0, %1, 0;" : "=l"(r) : "l"(p));
+        c = reinterpret_cast<PeelCounters *>(r);
+        p = reinterpret_cast<uint64_t>(&total);
+        asm("mapa.u64 %0, %1, 0;" : "=l"(r) : "l"(p));
+        tot = reinterpret_cast<unsigned *>(r);
+    }
+    sync();
+    PeelState st;
+    if (resume) {
+        st = a.ctl->st;
+    } else {
+        peel_setup(a, tid, nth, tot);
+        sync();
+        st = PeelState{0, 0, 0, -1, -1, *(volatile unsigned *)tot};
+    }
+    peel_rounds(a, c, st, 0, tid, nth, sync);
+    sync();  // the first CTA's shared memory outlives the others' last access
 }
 
 // Out-degree in the DAG u -> w iff (key[u], u) < (key[w], w), both alive.
@@ -897,15 +1024,23 @@ int launch_peel_update(const kcl_graph *g, Workspace &w, const uint32_t *fin, ui
 }
 
 constexpr int kPeelThreads = 1024;
+// Graphs up to this size are peeled in the cluster alone, and the grid leaves
+// the last kHandover vertices to it.  Orientation stage of the 1M-vertex and
+// the 262k-vertex R-MAT graph in ms: handover at 8k vertices 11.2 / 5.0, 32k
+// 10.4 / 3.6, 128k 9.2 / 3.2, 400k 9.3 / 3.2 (all cluster), the grid to the end
+// 10.4 / 5.4.
+constexpr uint32_t kClusterVertices = 1u << 17;
+constexpr uint64_t kClusterEntries = 1ull << 22;
+constexpr uint32_t kHandover = 1u << 17;
 
-// Blocks of the cooperative peel for n vertices: one per SM (fewer arrivals
-// per grid barrier), none beyond what n needs; -1 if it cannot be resident.
+// Blocks of the grid's peel for n vertices: one per SM (fewer arrivals per
+// grid barrier), none beyond what n needs; -1 if it cannot be resident.
 int peel_blocks(int num_sms, uint32_t n) {
     static std::atomic<int> cached{-1};  // several host threads (server slots) call this
     int per_sm = cached.load(std::memory_order_relaxed);
     if (per_sm < 0) {
         int b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_peel_coop, kPeelThreads, 0) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_peel_grid, kPeelThreads, 0) != cudaSuccess) {
             (void)cudaGetLastError();
             b = 0;
         }
@@ -919,26 +1054,68 @@ int peel_blocks(int num_sms, uint32_t n) {
     return blocks;
 }
 
-int launch_peel_coop(const kcl_graph *g, Workspace &w, PeelCtl *ctl, uint32_t *rl0, uint32_t *rl1,
-                     uint32_t *bl0, uint32_t *bl1, cudaStream_t s) {
-    int blocks = peel_blocks(g->num_sms, g->n);
-    if (blocks <= 0) return -1;
-    uint32_t n = g->n;
-    const uint64_t *rp = g->rp;
-    const uint32_t *col = g->col;
-    const uint8_t *alive = w.alive;
-    const uint32_t *cdeg = w.cdeg;
-    uint32_t *pdeg = w.peel_deg, *key = w.key, *fa = w.frontier_a, *fb = w.frontier_b;
-    // big rows: longer than 2048 and than 4x the mean degree, so there are at
-    // most nnz / big <= n / 4 of them (each list holds n / 2)
-    const uint64_t mean = n ? (g->nnz + n - 1) / n : 0;
-    uint64_t big = 4 * mean > 2048 ? 4 * mean : 2048;
-    void *args[] = {&n, (void *)&rp, (void *)&col, (void *)&alive, (void *)&cdeg, &pdeg, &key, &fa,
-                    &fb, &rl0, &rl1, &bl0, &bl1, &big, &ctl};
-    if (cudaLaunchCooperativeKernel((const void *)k_peel_coop, blocks, kPeelThreads, args, 0, s) !=
-        cudaSuccess)
-        return -1;
-    return 1;
+static void cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, int size, cudaStream_t s) {
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3((unsigned)size);
+    cfg.blockDim = dim3(kPeelThreads);
+    cfg.stream = s;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)size;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+}
+
+// Largest cluster of the peel the device can place (16 CTAs need the
+// non-portable size), 0 if none.
+static int peel_cluster_size() {
+    static std::atomic<int> cached{-1};
+    int best = cached.load(std::memory_order_relaxed);
+    if (best >= 0) return best;
+    best = 0;
+    (void)cudaFuncSetAttribute(k_peel_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (int size = 16; size >= 1 && !best; size >>= 1) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr;
+        cluster_config(cfg, attr, size, nullptr);
+        int fit = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit, k_peel_cluster, &cfg) == cudaSuccess && fit > 0) best = size;
+        (void)cudaGetLastError();
+    }
+    cached.store(best, std::memory_order_relaxed);
+    return best;
+}
+
+// The whole peel: wide rounds on the grid, the tail on one cluster.  The
+// control block is cleared first.  Returns the launches, -1 if it cannot run.
+static int peel_launches(PeelArgs a, int blocks, uint64_t nnz, cudaStream_t s) {
+    if (cudaMemsetAsync(a.ctl, 0, sizeof(PeelCtl), s) != cudaSuccess) return -1;
+    int size = peel_cluster_size();
+    const bool small = size && a.n <= kClusterVertices && nnz <= kClusterEntries;
+    int launches = 0;
+    if (!small) {
+        a.handover = size ? kHandover : 0;
+        void *args[] = {&a};
+        if (blocks <= 0 || cudaLaunchCooperativeKernel((const void *)k_peel_grid, blocks, kPeelThreads, args, 0, s) !=
+                               cudaSuccess)
+            return -1;
+        launches++;
+        if (!size) return launches;
+    } else {  // no more CTAs than 8 entries or one vertex a thread
+        const uint64_t work = std::max<uint64_t>(a.n, nnz / 8);
+        while (size > 1 && (uint64_t)(size / 2) * kPeelThreads >= work) size >>= 1;
+    }
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    cluster_config(cfg, attr, size, s);
+    if (cudaLaunchKernelEx(&cfg, k_peel_cluster, a, small ? 0 : 1) != cudaSuccess) return -1;
+    return launches + 1;
+}
+
+int launch_peel(const kcl_graph *g, Workspace &w, cudaStream_t s) {
+    const PeelArgs a{g->n, g->rp, g->col, w.alive, w.cdeg, reinterpret_cast<int *>(w.peel_deg), w.key,
+                     w.frontier_a, w.frontier_b, w.peel, 0};
+    return peel_launches(a, peel_blocks(g->num_sms, g->n), g->nnz, s);
 }
 
 int launch_orient(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s) {
@@ -976,8 +1153,8 @@ int launch_roots(const kcl_graph *g, uint32_t k, Workspace &w, uint32_t max_outd
 }  // namespace kcl
 
 // ======================================= allocation-free degeneracy ordering
-// Scratch of kcl_degeneracy_order_noalloc: peel degrees, two frontiers and the
-// control block of k_peel_coop for up to KCL_NOALLOC_MAX_VERTICES vertices.
+// Scratch of kcl_degeneracy_order_noalloc: peel degrees, the removal order, the
+// near list and the control block of the peel for up to KCL_NOALLOC_MAX_VERTICES vertices.
 // It is a fixed device array, so the call never allocates; in host code the
 // array's name is only a stand-in, and its device address is looked up with
 // cudaGetSymbolAddress once per device.
@@ -1036,30 +1213,11 @@ extern "C" kcl_status kcl_degeneracy_order_noalloc(uint32_t n, const uint64_t *r
     uint64_t need = ((uint64_t)n + kcl::kPeelThreads - 1) / kcl::kPeelThreads;
     if (need < (uint64_t)blocks) blocks = (int)need;
     cudaStream_t s = (cudaStream_t)stream;
-    uint32_t *pdeg = S;
-    uint32_t *fa = S + KCL_NOALLOC_MAX_VERTICES;
-    uint32_t *fb = S + 2 * (size_t)KCL_NOALLOC_MAX_VERTICES;
     kcl::PeelCtl *ctl = reinterpret_cast<kcl::PeelCtl *>(S + 3 * (size_t)KCL_NOALLOC_MAX_VERTICES);
-    // the control block keeps the previous call's contents: clear it (minv
-    // starts at all ones, everything else at zero)
-    if (cudaMemsetAsync(ctl, 0, sizeof(kcl::PeelCtl), s) != cudaSuccess ||
-        cudaMemsetAsync(ctl->minv, 0xFF, sizeof(ctl->minv), s) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return KCL_ECUDA;
-    }
-    uint32_t nn = n;
-    const uint64_t *rp = row_ptr;
-    const uint32_t *c = col;
-    const uint8_t *al = alive;
-    const uint32_t *deg = degree;
-    uint32_t *key = round_out;
-    uint32_t *rl0 = nullptr, *rl1 = nullptr;  // no room for remaining lists: full scans
-    uint32_t *bl0 = nullptr, *bl1 = nullptr;  // nor for big-row lists: a warp per frontier vertex
-    uint64_t big = ~0ull;
-    void *args[] = {&nn, (void *)&rp, (void *)&c, (void *)&al, (void *)&deg, &pdeg, &key, &fa, &fb,
-                    &rl0, &rl1, &bl0, &bl1, &big, &ctl};
-    if (cudaLaunchCooperativeKernel((const void *)kcl::k_peel_coop, blocks, kcl::kPeelThreads, args, 0, s) !=
-        cudaSuccess) {
+    const kcl::PeelArgs a{n, row_ptr, col, alive, degree, reinterpret_cast<int *>(S), round_out,
+                          S + KCL_NOALLOC_MAX_VERTICES, S + 2 * (size_t)KCL_NOALLOC_MAX_VERTICES, ctl, 0};
+    // the entry count is on the device: only small n goes to the cluster alone
+    if (kcl::peel_launches(a, blocks, n <= 1u << 15 ? 0 : ~0ull, s) < 0) {
         (void)cudaGetLastError();
         return KCL_ECUDA;
     }
