@@ -59,7 +59,7 @@ kcl_status dev_alloc(T **p, size_t count) {
 
 void free_workspace(Workspace &w) {
     void *ptrs[] = {w.alive, w.alive_core, w.cdeg, w.key, w.peel_deg, w.frontier_a, w.frontier_b,
-                    w.parent, w.comp_n, w.comp_sdeg, w.comp_flag, w.outdeg, w.optr, w.oadj,
+                    w.parent, w.comp_n, w.comp_flag, w.outdeg, w.take, w.optr, w.oadj,
                     w.roots, w.hist, w.scan_tmp, w.queue, w.members, w.comp_slot, w.arena, w.res,
                     w.peel, w.slots};
     for (void *p : ptrs)
@@ -97,7 +97,7 @@ kcl_status ensure_workspace(kcl_graph *g) {
     KCL_TRY(dev_alloc(&w.frontier_b, n));
     KCL_TRY(dev_alloc(&w.parent, n));
     KCL_TRY(dev_alloc(&w.comp_n, n));
-    KCL_TRY(dev_alloc(&w.comp_sdeg, n));
+    KCL_TRY(dev_alloc(&w.take, n));
     KCL_TRY(dev_alloc(&w.comp_flag, n));
     KCL_TRY(dev_alloc(&w.outdeg, n + 1));
     KCL_TRY(dev_alloc(&w.optr, n + 1));
@@ -249,15 +249,21 @@ kcl_status run_front(kcl_graph *g, uint32_t k, kcl_ordering ord, const kcl_ring 
     // ---- stage 0: Pre-Core
     T.begin(0);
     // without Pre-Core the threshold is 0: every vertex stays
-    T.add(0, launch_precore_init(g, (g->options & KCL_OPT_NO_PRECORE) ? 1u : k, w, s));
+    const uint32_t kcore = (g->options & KCL_OPT_NO_PRECORE) ? 1u : k;
     uint32_t *fa = w.frontier_a, *fb = w.frontier_b;
-    for (;;) {
-        uint32_t nin = 0;
-        KCL_TRY(read_u32(g, &w.res->frontier, &nin));
-        if (nin == 0) break;
-        KCL_TRY(set_u32(g, &w.res->frontier, 0));
-        T.add(0, launch_precore_round(g, k, fa, nin, fb, w, s));
-        std::swap(fa, fb);
+    if (const int l = launch_precore(g, kcore, w, s); l > 0) {
+        T.add(0, l);
+    } else {  // no co-resident launch here: one launch per round
+        (void)cudaGetLastError();
+        T.add(0, launch_precore_init(g, kcore, w, s));
+        for (;;) {
+            uint32_t nin = 0;
+            KCL_TRY(read_u32(g, &w.res->frontier, &nin));
+            if (nin == 0) break;
+            KCL_TRY(set_u32(g, &w.res->frontier, 0));
+            T.add(0, launch_precore_round(g, k, fa, nin, fb, w, s));
+            std::swap(fa, fb);
+        }
     }
     KCL_CK(cudaMemcpyAsync(w.alive_core, w.alive, n, cudaMemcpyDeviceToDevice, s));
     T.end(0);
@@ -276,12 +282,7 @@ kcl_status run_front(kcl_graph *g, uint32_t k, kcl_ordering ord, const kcl_ring 
     T.begin(2);
     if (ord == KCL_ORDER_DEGREE) {
         T.add(2, launch_degree_key(g, w, s));
-    } else if (run_peel(g, T)) {
-        uint32_t err = 0;
-        KCL_CK(cudaMemcpyAsync(&err, &w.peel->error, sizeof(err), cudaMemcpyDeviceToHost, s));
-        KCL_CK(cudaStreamSynchronize(s));
-        if (err) return KCL_ETIMEOUT;
-    } else {
+    } else if (!run_peel(g, T)) {
         T.add(2, launch_peel_init(g, w, s));
         uint32_t remaining = 0;
         KCL_TRY(read_u32(g, &w.res->remaining, &remaining));
@@ -311,14 +312,15 @@ kcl_status run_front(kcl_graph *g, uint32_t k, kcl_ordering ord, const kcl_ring 
     }
     KCL_CK(cudaMemsetAsync(&w.res->max_outdeg, 0, sizeof(unsigned), s));
     T.add(2, launch_orient(g, k, w, s));
-    KCL_TRY(read_u32(g, &w.res->max_outdeg, &fe.max_outdeg));
     uint32_t *limits = fe.limits;
     fe.n_classes = ord == KCL_ORDER_DEGREE ? sdegree_classes(limits, 16) : bitcol_classes(limits, 16);
-    T.add(2, launch_roots(g, k, w, fe.max_outdeg, fe.class_begin, limits, fe.n_classes, s));
+    T.add(2, launch_roots(g, k, w, limits, fe.n_classes, s));
     T.end(2);
     KCL_TRY(read_result(g));
+    if (w.h_res->peel_error) return KCL_ETIMEOUT;
+    fe.max_outdeg = w.h_res->max_outdeg;
     fe.n_roots = w.h_res->n_roots;
-    fe.class_begin[fe.n_classes] = fe.n_roots;
+    for (int c = 0; c <= fe.n_classes; c++) fe.class_begin[c] = w.h_res->class_begin[c];
     fe.pre_count = w.h_res->pre_count;
     if (w.h_res->status) return status_from_device(w.h_res->status);
     // roots above the largest class cannot be processed
@@ -880,7 +882,7 @@ kcl_status kcl_scratch_bytes(const kcl_graph *g, uint64_t *workspace, uint64_t *
         // mirrors ensure_workspace's allocations
         const uint64_t n = (uint64_t)w.n_cap + 1, half = w.nnz_cap / 2 + 1;
         ws = 2 * n                                  // alive, alive_core
-             + 4 * n * 13 + 8 * n                   // u32 arrays, comp_sdeg
+             + 4 * n * 13 + 8 * n                   // u32 arrays, take
              + 4 * 2                                // outdeg, optr extra entry
              + 4 * half                             // oadj
              + 4 * (3 * n + 1024) + 4 * (n / 1024 + 1024) + 4 * 64

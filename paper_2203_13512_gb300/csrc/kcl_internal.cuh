@@ -38,8 +38,9 @@ struct DevResult {
     unsigned int min_deg;            // minimum current degree (degeneracy peel)
     unsigned int remaining;          // vertices not yet peeled
     unsigned int n_clique_comps;     // components removed by Pre-List
-    unsigned int pad;
+    unsigned int peel_error;         // error word of Pre-Core's or the peel's barriers
     unsigned long long deadline_ns;  // %globaltimer value after which listing stops (0: none)
+    unsigned int class_begin[KCL_MAX_CLASSES + 1];  // root positions where the out-degree classes start
 };
 
 // Counters of the degeneracy peel's rounds (all zero at launch): frontier
@@ -69,6 +70,11 @@ struct PeelCtl {
     unsigned big[3][kPeelBig];
 };
 
+// Out-degree limits of the classes, passed by value.
+struct ClassLimits {
+    uint32_t d[KCL_MAX_CLASSES];
+};
+
 // One graph of a batch: its device CSR and its place in the disjoint union.
 struct BatchSrc {
     const uint64_t *rp;
@@ -92,9 +98,9 @@ struct Workspace {
     uint32_t *frontier_b = nullptr;  // n
     uint32_t *parent = nullptr;      // n: union-find forest (Pre-List)
     uint32_t *comp_n = nullptr;      // n: component sizes (by root)
-    unsigned long long *comp_sdeg = nullptr;  // n: component degree sums
     uint32_t *comp_flag = nullptr;   // n: 1 = clique component root
     uint32_t *outdeg = nullptr;      // n
+    unsigned long long *take = nullptr;  // n: which of a row's first 64 entries are out-neighbours
     uint32_t *optr = nullptr;        // n + 1: out-CSR offsets
     uint32_t *oadj = nullptr;        // nnz/2: out-neighbours, ascending id
     uint32_t *roots = nullptr;       // n: roots sorted by d+ descending
@@ -517,6 +523,9 @@ inline bool allow_max_smem(K kern) {
 // kcl_prep.cu
 int launch_validate(const kcl_graph *g, DevResult *res, cudaStream_t s);
 int launch_degrees(const kcl_graph *g, uint32_t *deg, cudaStream_t s);
+// All of Pre-Core in one launch of co-resident blocks (clears w.peel first); -1
+// if it cannot launch.
+int launch_precore(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s);
 int launch_precore_init(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s);
 int launch_precore_round(const kcl_graph *g, uint32_t k, const uint32_t *fin, uint32_t nin,
                          uint32_t *fout, Workspace &w, cudaStream_t s);
@@ -534,8 +543,8 @@ int launch_peel_min(const kcl_graph *g, Workspace &w, cudaStream_t s);
 // w.peel first); -1 if it cannot launch.
 int launch_peel(const kcl_graph *g, Workspace &w, cudaStream_t s);
 int launch_orient(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s);
-int launch_roots(const kcl_graph *g, uint32_t k, Workspace &w, uint32_t max_outdeg,
-                 uint32_t *class_begin, const uint32_t *class_limits, int n_classes,
+// Roots by descending out-degree; res->class_begin, n_roots and peel_error.
+int launch_roots(const kcl_graph *g, uint32_t k, Workspace &w, const uint32_t *class_limits, int n_classes,
                  cudaStream_t s);
 int launch_exclusive_scan(const uint32_t *in, uint32_t *out, uint32_t n, uint32_t *block_tmp,
                           cudaStream_t s);
