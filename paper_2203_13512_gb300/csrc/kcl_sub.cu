@@ -21,10 +21,11 @@
 //     once per (node, a) and a clique costs one SplitMix64 round (two when
 //     the root's own id is the largest) instead of k and a merge.
 // Listing kernels of the 1M-vertex R-MAT graph (16 edges a vertex), before and
-// now: k = 5 colour count 179.3 -> 47.1 ms, k = 4 colour listing 201.2 -> 111.7
-// ms (2.06e10 records, 2.96 TB/s of stores; the stores alone would take 49 ms at
+// now: k = 5 colour count 179.3 -> 42.2 ms, k = 4 colour listing 201.2 -> 101.8
+// ms (2.06e10 records, 3.2 TB/s of stores; the stores alone would take 49 ms at
 // the measured copy bandwidth).  Counting is bound by the ALU pipe, listing by
-// issue slots around the hash round.
+// issue slots around the hash round.  A kernel per k: with all of k = 3..6 in
+// one, 45.0 and 106.0 ms (registers, instruction cache).
 #include "kcl_internal.cuh"
 
 namespace kcl {
@@ -40,30 +41,39 @@ constexpr unsigned kFull = 0xffffffffu;
 __host__ __device__ inline uint32_t row_words4(uint32_t D) { return (((D + 31) >> 5) + 3) & ~3u; }
 __host__ __device__ inline uint32_t row_stride(uint32_t W) { return ((W >> 2) & 1) ? W : W + 4; }
 
-// Compact lower-triangular matrix: row i holds 4 (i / 128 + 1) words, so rows
-// are 16-byte aligned and the words above the diagonal's 128-bit group take no
-// room.
+// Compact lower-triangular matrix in groups of G words: row i holds
+// G (i / 32 G + 1) words, so rows are G-word aligned and most words above the
+// diagonal take no room.  Counting reads rows as 128-bit vectors (G = 4), listing
+// single words (G = 2, a third less room at 160 rows).
+template <int G>
 __host__ __device__ inline uint32_t tri_off(uint32_t i) {
-    const uint32_t R = i >> 7;
-    return 256 * R * (R + 1) + (i & 127u) * 4 * (R + 1);
+    const uint32_t R = i / (32 * G);
+    return 16 * G * G * R * (R + 1) + i % (32 * G) * G * (R + 1);
 }
-__host__ __device__ inline uint32_t tri_words(uint32_t c) { return tri_off((c + 31) & ~31u); }
+template <int G>
+__host__ __device__ inline uint32_t tri_words(uint32_t c) { return tri_off<G>((c + 31) & ~31u); }
+
+// Words a candidate set of c members takes in a warp's room: its ids (listing),
+// its matrix, and its index list (u16) at the end.
+__host__ __device__ inline uint32_t ids_words(uint32_t c, bool list) { return list ? (c + 3) & ~3u : 0u; }
+__host__ __device__ inline uint32_t idx_words(uint32_t c) { return ((c + 7) >> 3) << 2; }
+__host__ __device__ inline uint32_t set_room(uint32_t c, bool list) {
+    return ids_words(c, list) + (((list ? tri_words<2>(c) : tri_words<4>(c)) + 3) & ~3u) + idx_words(c);
+}
 
 // Shared memory of one subproblem (words).  RS, LEN, HK, HV, BM and the queues
 // belong to the build and are dead afterwards: the warps' scratch (X) overlays
 // them.  Per warp: kBitmaps candidate bitmaps of W words, the extract masks
-// (8 W), the index list (D u16) and the compact matrix with its ids (blob).
+// (8 W) and the room of the compacted set.
 constexpr uint32_t kBitmaps = 3;  // candidate sets of the path (k <= 6)
 constexpr uint32_t kQueue = 64;   // build: members found in a warp's out-lists, waiting for lookup
 struct Lay {
-    uint32_t D, W, WP, NBR, META, A, X, RS, LEN, HK, HV, BM, Q, per_warp, blob, total;
+    uint32_t D, W, WP, NBR, META, A, X, RS, LEN, HK, HV, BM, Q, per_warp, room, total;
 };
 
-__host__ __device__ inline uint32_t scratch_fixed(uint32_t D, uint32_t W) {
-    return (kBitmaps * W + 8 * W + D / 2 + 3) & ~3u;
-}
+__host__ __device__ inline uint32_t scratch_fixed(uint32_t W) { return (kBitmaps + 8) * W; }
 
-__host__ __device__ inline Lay make_lay(uint32_t D, uint32_t nw, uint32_t blob) {
+__host__ __device__ inline Lay make_lay(uint32_t D, uint32_t nw, uint32_t room) {
     Lay L;
     const uint32_t T = hash_cap(D);
     L.D = D;
@@ -79,8 +89,8 @@ __host__ __device__ inline Lay make_lay(uint32_t D, uint32_t nw, uint32_t blob) 
     L.HV = L.HK + T;            // hash values, u16
     L.BM = L.HV + T / 2;        // 16 T filter bits
     L.Q = L.BM + T / 2;         // per warp: kQueue ids, kQueue u16 rows
-    L.blob = blob;
-    L.per_warp = scratch_fixed(D, L.W) + blob;
+    L.room = room;
+    L.per_warp = scratch_fixed(L.W) + room;
     const uint32_t build = 2 * D + 2 * T + nw * (kQueue + kQueue / 2);
     const uint32_t walk = nw * L.per_warp;
     L.total = L.X + (((build > walk ? build : walk) + 3) & ~3u);
@@ -92,9 +102,9 @@ struct SubArgs {
     uint32_t begin, end;   // root positions of the class
     uint32_t parts;        // CTA form: a root's children are shared by this many units
     unsigned *queue;
-    uint32_t *gscratch;    // per-warp global blobs (larger candidate sets), gwords each
+    uint32_t *gscratch;    // per-warp room in global memory (larger candidate sets), gwords each
     uint32_t gwords;
-    uint32_t kmax, D, blob, dfs_warps;
+    uint32_t D, room, dfs_warps;
     uint32_t *ring;
     unsigned long long capacity;
     int wrap;
@@ -118,21 +128,20 @@ struct Group {
 
 // --------------------------------------------------------------- build
 // A batch of nb <= 32 queued (id, row) pairs: looks the id up in the table of
-// N+_u and records the edge.  SYM: both bits; else row max(i, j) gets bit
-// min(i, j); rows = false counts only.
-template <bool SYM>
+// N+_u and records the edge.
+enum Rows { kNoRows, kLower, kBoth };  // count only; row max(i, j) gets bit min(i, j); both bits
 __device__ __forceinline__ uint32_t link(const uint32_t *qid, const uint16_t *qrow, uint32_t nb,
                                          const uint32_t *hk, const uint16_t *hv, uint32_t T, uint32_t shift,
-                                         uint32_t *A, uint32_t WP, bool rows) {
+                                         uint32_t *A, uint32_t WP, Rows rows) {
     const unsigned lane = lane_id();
     uint32_t hit = 0;
     if (lane < nb) {
         const int x = hash_find(hk, hv, T, shift, qid[lane]);
         if (x >= 0) {
             hit = 1;
-            if (rows) {
+            if (rows != kNoRows) {
                 const uint32_t i = qrow[lane], j = (uint32_t)x;
-                if (SYM) {
+                if (rows == kBoth) {
                     atomicOr(&A[i * WP + (j >> 5)], 1u << (j & 31));
                     atomicOr(&A[j * WP + (i >> 5)], 1u << (i & 31));
                 } else {
@@ -154,9 +163,9 @@ __device__ __forceinline__ uint32_t link(const uint32_t *qid, const uint16_t *qr
 // they are short.  Testing every entry in the table itself, with the lists
 // flattened over the lanes by a search in their prefix sums, took 2.9x as long
 // (the k = 3 count of R-MAT 20: 27.6 ms).
-template <bool CTA, bool SYM>
+template <bool CTA>
 __device__ uint32_t build(uint32_t d, uint32_t base, const SubArgs &a, const Lay &L, uint32_t *S,
-                          bool rows) {
+                          Rows rows) {
     using G = Group<CTA>;
     const uint32_t tid = G::tid(), lane = lane_id(), warp = G::warp(), nw = G::size() >> 5;
     uint32_t *nbr = S + L.NBR, *rs = S + L.RS, *len = S + L.LEN, *hk = S + L.HK, *bm = S + L.BM, *A = S + L.A;
@@ -167,7 +176,7 @@ __device__ uint32_t build(uint32_t d, uint32_t base, const SubArgs &a, const Lay
     hash_size(d, &T, &hshift);
     for (uint32_t i = tid; i < T; i += G::size()) hk[i] = kHashEmpty;
     for (uint32_t i = tid; i < T / 2; i += G::size()) bm[i] = 0;
-    if (rows) {
+    if (rows != kNoRows) {
         uint4 *A4 = reinterpret_cast<uint4 *>(A);
         for (uint32_t i = tid; i < (d * L.WP) >> 2; i += G::size()) A4[i] = make_uint4(0, 0, 0, 0);
     }
@@ -223,7 +232,7 @@ __device__ uint32_t build(uint32_t d, uint32_t base, const SubArgs &a, const Lay
                 pend += __popc(bal);
                 if (pend >= 32) {
                     __syncwarp();
-                    hits += link<SYM>(qid, qrow, 32, hk, hv, T, hshift, A, L.WP, rows);
+                    hits += link(qid, qrow, 32, hk, hv, T, hshift, A, L.WP, rows);
                     __syncwarp();
                     pend -= 32;
                     if (lane < pend) {
@@ -236,7 +245,7 @@ __device__ uint32_t build(uint32_t d, uint32_t base, const SubArgs &a, const Lay
         }
     }
     __syncwarp();
-    hits += link<SYM>(qid, qrow, pend, hk, hv, T, hshift, A, L.WP, rows);
+    hits += link(qid, qrow, pend, hk, hv, T, hshift, A, L.WP, rows);
     G::sync();
     return hits;
 }
@@ -246,17 +255,19 @@ __device__ uint32_t build(uint32_t d, uint32_t base, const SubArgs &a, const Lay
 struct Scratch {
     uint32_t *cb;      // kBitmaps candidate bitmaps, W words each
     uint32_t *masks;   // extract masks, 8 words per bitmap word
-    uint16_t *idx;     // members of the compacted set
-    uint32_t *blob;    // compact matrix (listing: ids first) in shared memory
-    uint32_t blob_cap;
-    uint32_t *gblob;   // the same in global memory for larger sets
+    uint32_t *mem;     // room of the compacted set: ids, matrix, index list at the end
+    uint32_t room;
+    uint32_t *gmem;    // ids and matrix of larger sets, in global memory
+    __device__ __forceinline__ uint16_t *idx(uint32_t c, bool fits) const {
+        return reinterpret_cast<uint16_t *>(fits ? mem + room - idx_words(c) : mem);
+    }
 };
 
-// Members of the bitmap C (nw words) in ascending order.
-__device__ __forceinline__ void index_list(const uint32_t *C, uint32_t nw, uint16_t *idx) {
+// Members of the bitmap C (words w0 .. nw - 1) in ascending order.
+__device__ __forceinline__ void index_list(const uint32_t *C, uint32_t w0, uint32_t nw, uint16_t *idx) {
     const unsigned lane = lane_id(), lt = (1u << lane) - 1u;
     uint32_t base = 0;
-    for (uint32_t t = 0; t < nw; t++) {
+    for (uint32_t t = w0; t < nw; t++) {
         const uint32_t m = C[t];
         if ((m >> lane) & 1u) idx[base + __popc(m & lt)] = (uint16_t)(t * 32 + lane);
         base += __popc(m);
@@ -297,23 +308,33 @@ __device__ __forceinline__ void extract_masks(const uint32_t *C, uint32_t nw, ui
 __device__ __forceinline__ uint32_t pick(uint32_t sel, uint32_t a, uint32_t b) { return (sel & a) | (~sel & b); }
 
 // The rows of C's members restricted to C, as a lower-triangular bit matrix
-// over C's own indices (bits below the diagonal; out: tri_words(c) words).
-// 32 rows at a time, a lane per row: the row's words are read as 128-bit
-// vectors, each is extracted by C's masks and appended to the lane's output;
-// all lanes append the same number of bits, so the bookkeeping is uniform.
-// Returns the lane's number of set bits.
+// over C's own indices (bits below the diagonal).  32 rows at a time, a lane per
+// row: the row's words are read as 128-bit vectors, each is extracted by C's
+// masks and appended to the lane's output; all lanes append the same number of
+// bits, so the bookkeeping is uniform.  Returns the lane's number of set bits.
+template <int G>
 __device__ uint32_t compact(const uint32_t *A, uint32_t WP, uint32_t c, const uint32_t *masks,
                             const uint16_t *idx, uint32_t *out) {
     const unsigned lane = lane_id(), lt = (1u << lane) - 1u;
+    const uint32_t tbeg = (idx[0] >> 7) << 2;
     uint32_t sum = 0;
     for (uint32_t r = 0; r * 32 < c; r++) {
         const uint32_t i = r * 32 + lane;
         const bool act = i < c;
         const uint4 *row = reinterpret_cast<const uint4 *>(A + (uint32_t)idx[act ? i : c - 1] * WP);
         const uint32_t tend = (idx[min(r * 32 + 31, c - 1)] >> 5) + 1;
-        uint32_t *o = out + tri_off(i);
+        uint32_t *o = out + tri_off<G>(i);
         uint32_t lo = 0, ow = 0, sh = 0;
-        for (uint32_t t0 = 0; t0 < tend; t0 += 4) {
+        auto put = [&]() {  // the next output word; words above the diagonal are dropped
+            if (ow <= r) {
+                uint32_t w = act ? lo : 0u;
+                if (ow == r) w &= lt;
+                o[ow] = w;
+                sum += __popc(w);
+            }
+            ow++;
+        };
+        for (uint32_t t0 = tbeg; t0 < tend; t0 += 4) {
             const uint4 v = row[t0 >> 2];
 #pragma unroll
             for (uint32_t z = 0; z < 4; z++) {
@@ -332,23 +353,12 @@ __device__ uint32_t compact(const uint32_t *A, uint32_t WP, uint32_t c, const ui
                 sh += m1.y;
                 if (sh >= 32) {
                     sh -= 32;
-                    if (ow <= r) {
-                        uint32_t w = act ? lo : 0u;
-                        if (ow == r) w &= lt;
-                        o[ow] = w;
-                        sum += __popc(w);
-                    }
-                    ow++;
+                    put();
                     lo = __funnelshift_rc(x, 0u, m1.y - sh);  // the m1.y - sh bits already stored leave
                 }
             }
         }
-        if (ow <= r) {
-            uint32_t w = act ? lo : 0u;
-            if (ow == r) w &= lt;
-            o[ow] = w;
-            sum += __popc(w);
-        }
+        if (ow <= r) put();
     }
     __syncwarp();
     return sum;
@@ -370,30 +380,32 @@ __device__ __forceinline__ uint32_t lop_maj(uint32_t a, uint32_t b, uint32_t c) 
     asm("lop3.b32 %0, %1, %2, %3, 0xE8;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
     return r;
 }
-
 // Rows p0..p1 (both even) against the lanes' rows (words 4 g .. 4 g + NWD - 1
 // of row q in qv): lane q adds |row(q) & row(p)| over those words when bit q
 // of row p is set (word b of row p; LAST: b is the group's last word).  Bits
 // are summed through a carry-save adder, two rows at a time: POPC runs at a
 // quarter of LOP3's rate and is needed only for the carries (weight 2).
-template <int NWD, bool LAST>
+template <int NWD, bool LAST, int UNROLL>
 __device__ __forceinline__ void tri_rows(const uint32_t *M, uint32_t b, uint32_t g, uint32_t p0, uint32_t p1,
                                          const uint4 &qv, uint32_t &ones, uint32_t &twos) {
-    const uint32_t up = 31u - lane_id();
+    // 2^(31 - lane), opaque to the compiler: moving bit `lane` to the sign is
+    // then a multiply, off the ALU pipe that bounds this loop
+    uint32_t up;
+    asm("shl.b32 %0, %1, %2;" : "=r"(up) : "r"(1u), "r"(31u - lane_id()));
     const uint32_t q[4] = {qv.x, qv.y, qv.z, qv.w};
     for (uint32_t p = p0; p < p1;) {
         const uint32_t R = p >> 7, stride = 4 * (R + 1);
         const uint32_t end = min(p1, (R + 1) << 7);
-        const uint32_t *rp = M + tri_off(p) + 4 * g;
-#pragma unroll 2
+        const uint32_t *rp = M + tri_off<4>(p) + 4 * g;
+#pragma unroll UNROLL
         for (; p < end; p += 2, rp += 2 * stride) {
             const uint4 av = *reinterpret_cast<const uint4 *>(rp);
             const uint4 bv = *reinterpret_cast<const uint4 *>(rp + stride);
             const uint32_t x[4] = {av.x, av.y, av.z, av.w}, y[4] = {bv.x, bv.y, bv.z, bv.w};
             const uint32_t ea = LAST ? x[NWD - 1] : rp[b - 4 * g];
             const uint32_t eb = LAST ? y[NWD - 1] : rp[stride + b - 4 * g];
-            const uint32_t ma = (uint32_t)((int32_t)(ea << up) >> 31);
-            const uint32_t mb = (uint32_t)((int32_t)(eb << up) >> 31);
+            const uint32_t ma = (uint32_t)((int32_t)(ea * up) >> 31);
+            const uint32_t mb = (uint32_t)((int32_t)(eb * up) >> 31);
 #pragma unroll
             for (int w = 0; w < NWD; w++) {
                 const uint32_t s = lop_and3(q[w], x[w], ma), t = lop_and3(q[w], y[w], mb);
@@ -405,21 +417,22 @@ __device__ __forceinline__ void tri_rows(const uint32_t *M, uint32_t b, uint32_t
 }
 
 // Triangles of the compact matrix M over c vertices (lane's share).
+template <int UNROLL>
 __device__ uint32_t tri_matrix(const uint32_t *M, uint32_t c) {
     const unsigned lane = lane_id();
     const uint32_t nb = (c + 31) >> 5, rows = (c + 1) & ~1u;
     uint32_t ones = 0, twos = 0;
     for (uint32_t b = 0; b < nb; b++) {
-        const uint32_t *rq = M + tri_off(b * 32 + lane);
+        const uint32_t *rq = M + tri_off<4>(b * 32 + lane);
         const uint32_t last = b >> 2;
         for (uint32_t g = 0; g < last; g++)
-            tri_rows<4, false>(M, b, g, b * 32, rows, *reinterpret_cast<const uint4 *>(rq + 4 * g), ones, twos);
+            tri_rows<4, false, UNROLL>(M, b, g, b * 32, rows, *reinterpret_cast<const uint4 *>(rq + 4 * g), ones, twos);
         const uint4 qv = *reinterpret_cast<const uint4 *>(rq + 4 * last);
         switch (b & 3) {
-            case 0: tri_rows<1, true>(M, b, last, b * 32, rows, qv, ones, twos); break;
-            case 1: tri_rows<2, true>(M, b, last, b * 32, rows, qv, ones, twos); break;
-            case 2: tri_rows<3, true>(M, b, last, b * 32, rows, qv, ones, twos); break;
-            default: tri_rows<4, true>(M, b, last, b * 32, rows, qv, ones, twos);
+            case 0: tri_rows<1, true, UNROLL>(M, b, last, b * 32, rows, qv, ones, twos); break;
+            case 1: tri_rows<2, true, UNROLL>(M, b, last, b * 32, rows, qv, ones, twos); break;
+            case 2: tri_rows<3, true, UNROLL>(M, b, last, b * 32, rows, qv, ones, twos); break;
+            default: tri_rows<4, true, UNROLL>(M, b, last, b * 32, rows, qv, ones, twos);
         }
     }
     return 2 * twos + __popc(ones);
@@ -433,10 +446,12 @@ __device__ uint32_t tri_count(const uint32_t *A, uint32_t WP, const uint32_t *C,
                               const Scratch &sc) {
     const unsigned lane = lane_id();
     if (c < 3) return 0;
-    index_list(C, nw, sc.idx);
+    const bool fits = set_room(c, false) <= sc.room;
+    uint16_t *idx = sc.idx(c, fits);
+    index_list(C, 0, nw, idx);
     if (c <= 32) {
         // lanes beyond c look at the last member's bit, zero in every row
-        const uint32_t me = sc.idx[min(lane, c - 1)];
+        const uint32_t me = idx[min(lane, c - 1)];
         const uint32_t *col = A + (me >> 5);
         const uint32_t sh = me & 31u;
         uint32_t mine = 0, acc = 0;
@@ -453,12 +468,12 @@ __device__ uint32_t tri_count(const uint32_t *A, uint32_t WP, const uint32_t *C,
     }
     extract_masks(C, nw, sc.masks);
     uint32_t acc;
-    if (tri_words(c) <= sc.blob_cap) {
-        compact(A, WP, c, sc.masks, sc.idx, sc.blob);
-        acc = tri_matrix(sc.blob, c);
+    if (fits) {
+        compact<4>(A, WP, c, sc.masks, idx, sc.mem);
+        acc = tri_matrix<2>(sc.mem, c);
     } else {
-        compact(A, WP, c, sc.masks, sc.idx, sc.gblob);
-        acc = tri_matrix(sc.gblob, c);
+        compact<4>(A, WP, c, sc.masks, idx, sc.gmem);
+        acc = tri_matrix<2>(sc.gmem, c);
     }
     __syncwarp();
     return acc;
@@ -471,13 +486,14 @@ __device__ uint32_t pair_count(const uint32_t *A, uint32_t WP, const uint32_t *C
                                const Scratch &sc) {
     const unsigned lane = lane_id();
     if (c < 2) return 0;
-    index_list(C, nw, sc.idx);
+    uint16_t *idx = sc.idx(c, false);
+    index_list(C, 0, nw, idx);
     uint32_t acc = 0;
     const uint4 *c4 = reinterpret_cast<const uint4 *>(C);
     for (uint32_t i0 = 0; i0 < c; i0 += 32) {
         const uint32_t i = i0 + lane;
-        const uint32_t p = sc.idx[min(i, c - 1)];
-        const uint32_t nc = ((uint32_t)sc.idx[min(i0 + 31, c - 1)] >> 7) + 1;
+        const uint32_t p = idx[min(i, c - 1)];
+        const uint32_t nc = ((uint32_t)idx[min(i0 + 31, c - 1)] >> 7) + 1;
         const uint4 *row = reinterpret_cast<const uint4 *>(A + p * WP);
         uint32_t x = 0;
         for (uint32_t t = 0; t < nc; t++) {
@@ -552,7 +568,7 @@ __device__ __forceinline__ void list_rows(const uint32_t *M, uint32_t WP, uint32
         const uint32_t bl = b0 + lane * bstep;
         uint32_t mw = 0, idw = 0;
         if (bl < bend) {
-            mw = M[(DIRECT ? bl * WP : tri_off(bl)) + t];
+            mw = M[(DIRECT ? bl * WP : tri_off<2>(bl)) + t];
             if (DIRECT && (bl >> 5) == t) mw &= (1u << (bl & 31)) - 1u;
             idw = cid[bl];
         }
@@ -658,28 +674,28 @@ __device__ __forceinline__ void list_by_mode(const uint32_t *M, uint32_t WP, uin
 
 // Level-2 node: lists the cliques closed by the edges of G_u within C.
 template <int K>
-__device__ void list_node(const uint32_t *A, uint32_t WP, const uint32_t *C, uint32_t nw, uint32_t c,
+__device__ void list_node(const uint32_t *A, uint32_t WP, const uint32_t *C, uint32_t w0, uint32_t nw, uint32_t c,
                           const uint32_t *nbr, uint32_t ru, const uint32_t *path, uint32_t u,
                           const Scratch &sc, const SubArgs &a, unsigned long long &cnt,
                           unsigned long long &cks) {
     const unsigned lane = lane_id();
-    index_list(C, nw, sc.idx);
+    const bool fits = set_room(c, true) <= sc.room;
+    uint16_t *idx = sc.idx(c, fits);
+    index_list(C, w0, nw, idx);
     extract_masks(C, nw, sc.masks);
-    const uint32_t ids = (c + 3) & ~3u;
-    const bool shared = ids + tri_words(c) <= sc.blob_cap;
-    // members with an id below u: those with an index below ru
-    uint32_t cu = 0;
-    uint32_t *blob = shared ? sc.blob : sc.gblob;
+    uint32_t *ids = fits ? sc.mem : sc.gmem;
+    uint32_t *M = ids + ids_words(c, true);
+    uint32_t cu = 0;  // members with an id below u: those with an index below ru
     for (uint32_t i = lane; i < c; i += 32) {
-        const uint32_t x = sc.idx[i];
+        const uint32_t x = idx[i];
         cu += x < ru ? 1u : 0u;
-        blob[i] = nbr[x];
+        ids[i] = nbr[x];
     }
     cu = __reduce_add_sync(kFull, cu);
-    const uint32_t mine = compact(A, WP, c, sc.masks, sc.idx, blob + ids);
+    const uint32_t mine = compact<2>(A, WP, c, sc.masks, idx, M);
     cnt += mine;
     const uint32_t total = __reduce_add_sync(kFull, mine);
-    if (total) list_by_mode<K, false>(blob + ids, 0, c, blob, cu, path, u, 1, 1, a, total, cks);
+    if (total) list_by_mode<K, false>(M, 0, c, ids, cu, path, u, 1, 1, a, total, cks);
     __syncwarp();
 }
 
@@ -691,15 +707,15 @@ struct Sub {
 };
 
 // Candidate set of path vertex w below C (C null: all of N+_u): row(w) & C,
-// restricted to indices above w when rows are symmetric.  Returns its size.
-template <bool LIST>
+// restricted to indices above w when rows are symmetric (UP).  Returns its size.
+template <bool UP>
 __device__ __forceinline__ uint32_t next_set(const Sub &s, const uint32_t *C, uint32_t w, uint32_t *out) {
     const unsigned lane = lane_id();
     uint32_t x = 0;
     if (lane < s.W) {
         x = s.A[w * s.WP + lane];
         if (C) x &= C[lane];
-        if (LIST) {
+        if (UP) {
             if (lane < (w >> 5)) x = 0;
             else if (lane == (w >> 5)) x &= ~((2u << (w & 31)) - 1u);
         }
@@ -709,30 +725,27 @@ __device__ __forceinline__ uint32_t next_set(const Sub &s, const uint32_t *C, ui
     return __reduce_add_sync(kFull, __popc(x));
 }
 
-// Words that can be non-zero in a set below path vertex w: rows hold bits
-// below w (counting) or any (listing).
-template <bool LIST>
-__device__ __forceinline__ uint32_t set_words(const Sub &s, uint32_t w) {
-    return LIST ? (s.d + 31) >> 5 : (w >> 5) + 1;
-}
-
-// The subtree of a node with J path vertices below the root and candidate
-// set C (bitmap J - 1, c members).  Counting ends in tri_count at level 3 (J =
-// K - 4) or pair_count (K = 4), listing in list_node at level 2 (J = K - 3).
+// The subtree of a node with J path vertices below the root, the last one
+// `last`, and candidate set C (bitmap J - 1, c members).  Counting ends in
+// tri_count at level 3 (J = K - 4) or pair_count (K = 4), listing in list_node at
+// level 2 (J = K - 3).
 template <int K, int J, bool LIST>
 __device__ void walk(const Sub &s, uint32_t last, uint32_t c, uint32_t *path, const Scratch &sc,
                      const SubArgs &a, unsigned long long &cnt, unsigned long long &cks) {
     const uint32_t *C = sc.cb + (J - 1) * s.W;
-    const uint32_t nw = set_words<LIST>(s, last);
+    // words that can be non-zero: rows hold bits below the diagonal (counting),
+    // or both sides and a path ascends (listing)
+    const uint32_t w0 = LIST ? last >> 5 : 0u;
+    const uint32_t nw = LIST ? (s.d + 31) >> 5 : (last >> 5) + 1;
     if constexpr (LIST && J == K - 3) {
-        list_node<K>(s.A, s.WP, C, nw, c, s.nbr, s.ru, path, s.u, sc, a, cnt, cks);
+        list_node<K>(s.A, s.WP, C, w0, nw, c, s.nbr, s.ru, path, s.u, sc, a, cnt, cks);
     } else if constexpr (!LIST && K == 4) {
         cnt += pair_count(s.A, s.WP, C, nw, c, sc);
     } else if constexpr (!LIST && J == K - 4) {
         cnt += tri_count(s.A, s.WP, C, nw, c, sc);
     } else {
         uint32_t *Cn = sc.cb + J * s.W;
-        for (uint32_t t = 0; t < nw; t++) {
+        for (uint32_t t = w0; t < nw; t++) {
             uint32_t m = C[t];
             while (m) {
                 const uint32_t w = t * 32 + (__ffs(m) - 1);
@@ -785,23 +798,24 @@ __device__ __forceinline__ void attribute(unsigned long long mine, unsigned long
 // CTA: one root (or one of `parts` shares of its children) per CTA, built by
 // all warps, first-level children handed out to the warps, the ones with the
 // most candidates first.  Else one root per warp.
-template <bool CTA, bool LIST>
+// KK: the launch's k, or 0 for a batch whose roots have their own (a kernel per
+// k keeps each one's code, and its share of the instruction cache, to its leaf).
+template <bool CTA, bool LIST, int KK>
 __device__ __forceinline__ void run(const SubArgs &a) {
     extern __shared__ __align__(16) uint32_t smem[];
     using G = Group<CTA>;
     const unsigned lane = lane_id();
     const uint32_t wib = threadIdx.x >> 5, nwarps = CTA ? blockDim.x >> 5 : 1u;
-    const Lay L = make_lay(a.D, nwarps, a.blob);
+    const Lay L = make_lay(a.D, nwarps, a.room);
     uint32_t *S = CTA ? smem : smem + wib * L.total;
     uint32_t *meta = S + L.META;
     uint32_t *x = S + L.X + (CTA ? wib * L.per_warp : 0u);
     Scratch sc;
     sc.cb = x;
     sc.masks = x + kBitmaps * L.W;
-    sc.idx = reinterpret_cast<uint16_t *>(sc.masks + 8 * L.W);
-    sc.blob = x + scratch_fixed(L.D, L.W);
-    sc.blob_cap = L.blob;
-    sc.gblob = a.gscratch + (size_t)(blockIdx.x * (blockDim.x >> 5) + wib) * a.gwords;
+    sc.mem = x + scratch_fixed(L.W);
+    sc.room = L.room;
+    sc.gmem = a.gscratch + (size_t)(blockIdx.x * (blockDim.x >> 5) + wib) * a.gwords;
     const uint32_t units = (a.end - a.begin) * a.parts;
     const uint32_t nd = CTA && a.dfs_warps && a.dfs_warps < nwarps ? a.dfs_warps : nwarps;
     const unsigned long long deadline = __ldcg(&a.res->deadline_ns);
@@ -822,13 +836,14 @@ __device__ __forceinline__ void run(const SubArgs &a) {
         if (unit >= units) break;
         const uint32_t part = unit % a.parts;
         const uint32_t u = a.roots[a.begin + unit / a.parts];
-        const uint32_t k = a.kmap ? (uint32_t)a.kmap[u] : a.kmax;
+        const uint32_t k = KK ? (uint32_t)KK : (uint32_t)a.kmap[u];
         const uint32_t base = a.optr[u], d = a.optr[u + 1] - base;
         const unsigned long long before = cnt, before_cks = cks;
         // a k = 3 root has no children to share: its first unit does all of it
         const bool skip = k == 3 && part > 0;
         if (!skip) {
-            const uint32_t hits = build<CTA, LIST>(d, base, a, L, S, LIST || k > 3);
+            const Rows rows = LIST ? kBoth : k > 3 ? kLower : kNoRows;
+            const uint32_t hits = build<CTA>(d, base, a, L, S, rows);
             Sub s{S + L.A, S + L.NBR, L.WP, L.W, d, u, 0u, deadline};
             if (LIST) {
                 uint32_t below = 0;  // members with an id below u
@@ -845,8 +860,7 @@ __device__ __forceinline__ void run(const SubArgs &a) {
                 if (LIST) list_edges(s, G::warp(), nwarps, a, cnt, cks);
                 else cnt += hits;
             } else if (G::warp() < nd) {
-                // the part's children: counting takes the largest indices first
-                // (rows hold smaller ones), listing the smallest
+                // the part's children, the ones with the most candidates first
                 const uint32_t nch = part < d ? (d - 1 - part) / a.parts + 1 : 0u;
                 uint32_t i = 0;
                 for (;; i++) {
@@ -876,12 +890,13 @@ __device__ __forceinline__ void run(const SubArgs &a) {
     }
 }
 
-template <bool LIST>
+template <bool LIST, int KK>
 __global__ void __launch_bounds__(512, 2) k_sub_cta(const __grid_constant__ SubArgs a) {
-    run<true, LIST>(a);
+    run<true, LIST, KK>(a);
 }
+template <int KK>
 __global__ void __launch_bounds__(128, 8) k_sub_warp(const __grid_constant__ SubArgs a) {
-    run<false, false>(a);
+    run<false, false, KK>(a);
 }
 
 // -------------------------------------------------------------- host side
@@ -892,9 +907,9 @@ constexpr size_t kHalfSM = 112 * 1024;  // two CTAs per SM
 constexpr size_t kFullSM = 220 * 1024;
 
 struct Cfg {
-    uint32_t D, warps, blob, gwords;
+    uint32_t D, warps, room, gwords;
     size_t smem;
-    uint32_t per_sm;  // CTAs per SM the scratch is sized for
+    uint32_t per_sm;  // CTAs per SM the global room is sized for
 };
 
 // Launch shape of class c for a largest out-degree maxd.
@@ -904,33 +919,33 @@ Cfg config(int c, uint32_t maxd, bool listing) {
     f.D = (d + 31) & ~31u;
     if (f.D < 32) f.D = 32;
     const bool cta = listing || c >= kWarpClasses;
-    const uint32_t full = tri_words(f.D) + (listing ? f.D : 0u);
-    const uint32_t fixed = scratch_fixed(f.D, row_words4(f.D));
+    const uint32_t full = set_room(f.D, listing);
+    const uint32_t least = idx_words(f.D), fixed = scratch_fixed(row_words4(f.D));
     if (!cta) {
         f.warps = 4;  // warps per block, one root each
-        f.blob = full;
+        f.room = full;
         f.smem = 4 * (size_t)make_lay(f.D, 1, full).total * 4;
         f.gwords = 0;
         f.per_sm = 0;
         return f;
     }
     f.warps = f.D <= 128 ? 4 : f.D <= 256 ? 8 : 16;
-    const uint32_t resident = 32 / f.warps;  // 64 registers a thread: 1024 threads per SM
+    f.per_sm = 32 / f.warps;  // 64 registers a thread: 1024 threads per SM
     const uint32_t head = make_lay(f.D, 0, 0).X;
-    auto blob_in = [&](size_t cap) {
+    auto room_in = [&](size_t cap) {
         const uint32_t words = (uint32_t)(cap / 4);
-        const uint32_t room = words > head ? (words - head) / f.warps : 0u;
-        const uint32_t b = room > fixed ? (room - fixed) & ~3u : 0u;
+        const uint32_t each = words > head ? (words - head) / f.warps : 0u;
+        uint32_t b = each > fixed ? (each - fixed) & ~3u : 0u;
+        if (b < least) b = least;
         return b < full ? b : full;
     };
-    f.per_sm = resident;
-    f.blob = blob_in(f.D <= 256 ? kFullSM / resident - 1024 : kHalfSM);
-    if (f.D > 256 && f.blob < 512 && f.blob < full) {  // large rows: one CTA with room for its matrices
-        f.per_sm = 1;
-        f.blob = blob_in(kFullSM);
+    f.room = room_in(f.D <= 256 ? kFullSM / f.per_sm - 1024 : kHalfSM);
+    if (f.D > 256 && ((f.room < 512 && f.room < full) || make_lay(f.D, f.warps, f.room).total * 4 > kHalfSM)) {
+        f.per_sm = 1;  // large rows: one CTA with room for its matrices
+        f.room = room_in(kFullSM);
     }
-    f.smem = (size_t)make_lay(f.D, f.warps, f.blob).total * 4;
-    f.gwords = f.blob < full ? full : 0;
+    f.smem = (size_t)make_lay(f.D, f.warps, f.room).total * 4;
+    f.gwords = f.room < full ? full : 0;
     return f;
 }
 
@@ -966,9 +981,8 @@ int launch_sub(const kcl_graph *g, uint32_t k, Workspace &w, int c, uint32_t beg
     a.queue = queue;
     a.gscratch = w.arena;
     a.gwords = f.gwords;
-    a.kmax = k;
     a.D = f.D;
-    a.blob = f.blob;
+    a.room = f.room;
     a.dfs_warps = dfs_warps;
     a.ring = la.ring;
     a.capacity = la.capacity;
@@ -981,23 +995,29 @@ int launch_sub(const kcl_graph *g, uint32_t k, Workspace &w, int c, uint32_t beg
     const bool cta = la.listing || c >= kWarpClasses;
     int occ = 0;
     uint32_t n = end - begin;
+    using Kernel = void (*)(const SubArgs);
+    static const Kernel warp_kernels[] = {k_sub_warp<0>, k_sub_warp<3>, k_sub_warp<4>, k_sub_warp<5>, k_sub_warp<6>};
+    static const Kernel cta_kernels[2][5] = {
+        {k_sub_cta<false, 0>, k_sub_cta<false, 3>, k_sub_cta<false, 4>, k_sub_cta<false, 5>, k_sub_cta<false, 6>},
+        {k_sub_cta<true, 0>, k_sub_cta<true, 3>, k_sub_cta<true, 4>, k_sub_cta<true, 5>, k_sub_cta<true, 6>}};
+    const uint32_t ki = w.kmap ? 0u : k - 2;
+    const Kernel kern = cta ? cta_kernels[la.listing ? 1 : 0][ki] : warp_kernels[ki];
     if (!cta) {
-        if (!allow_max_smem(k_sub_warp) ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sub_warp, f.warps * 32, f.smem) != cudaSuccess)
+        if (!allow_max_smem(kern) ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, f.warps * 32, f.smem) != cudaSuccess)
             (void)cudaGetLastError();
         if (occ < 1) occ = 1;
         uint32_t blocks = (uint32_t)g->num_sms * occ;
         const uint32_t need = (n + f.warps - 1) / f.warps;
         if (blocks > need) blocks = need;
-        k_sub_warp<<<blocks, f.warps * 32, f.smem, s>>>(a);
+        kern<<<blocks, f.warps * 32, f.smem, s>>>(a);
         return 1;
     }
-    auto kern = la.listing ? k_sub_cta<true> : k_sub_cta<false>;
     if (!allow_max_smem(kern) ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, f.warps * 32, f.smem) != cudaSuccess)
         (void)cudaGetLastError();
     if (occ < 1) occ = 1;
-    if (occ > (int)f.per_sm) occ = (int)f.per_sm;  // global blobs per SM
+    if (occ > (int)f.per_sm) occ = (int)f.per_sm;  // global room per SM
     uint32_t blocks = (uint32_t)g->num_sms * occ;
     // a class with few roots shares each root's children over several CTAs,
     // which all build it
