@@ -28,6 +28,32 @@ __device__ __forceinline__ uint32_t warp_global() {
 }
 __device__ __forceinline__ uint32_t warps_total() { return (gridDim.x * blockDim.x) >> 5; }
 
+__device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t *smem, uint32_t *total) {
+    const unsigned lane = lane_id(), wid = threadIdx.x >> 5;
+    uint32_t v = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= (unsigned)o) v += y;
+    }
+    if (lane == 31) smem[wid] = v;
+    __syncthreads();
+    if (wid == 0) {
+        uint32_t s = lane < (blockDim.x >> 5) ? smem[lane] : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= (unsigned)o) s += y;
+        }
+        smem[lane] = s;
+    }
+    __syncthreads();
+    uint32_t warp_prefix = wid ? smem[wid - 1] : 0;
+    *total = smem[(blockDim.x >> 5) - 1];
+    __syncthreads();
+    return warp_prefix + v - x;
+}
+
 // ----------------------------------------------------------- validation
 // Row u: strictly ascending, ids < n, no self-loop, and every v in row u has
 // u in row v (binary search).  Also records the maximum degree.
@@ -541,6 +567,7 @@ __global__ void k_peel_update(const uint64_t *__restrict__ rp, const uint32_t *_
 constexpr int kNear = 32;                 // thresholds a near list covers
 constexpr uint32_t kBigRow = 4096;        // longer rows are walked by all warps
 constexpr int kGone = -(1 << 30);         // degree of a vertex that is not alive
+constexpr int kPeelThreads = 1024;
 
 struct PeelArgs {
     uint32_t n;
@@ -561,12 +588,25 @@ struct GridSync {
     unsigned nblocks;
     __device__ __forceinline__ bool operator()() const { return grid_barrier(ctl, nblocks); }
 };
+struct BlockSync {
+    __device__ __forceinline__ bool operator()() const {
+        __syncthreads();
+        return true;
+    }
+};
 struct ClusterSync {
     __device__ __forceinline__ bool operator()() const {
         asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
         return true;
     }
 };
+
+// Words other threads of the group write: from L2, or from shared memory (SH).
+template <bool SH, typename T>
+__device__ __forceinline__ T peel_load(const T *p) {
+    if constexpr (SH) return *reinterpret_cast<const volatile T *>(p);
+    else return __ldcg(p);
+}
 
 // Degrees, keys and the number of vertices to peel.
 __device__ void peel_setup(const PeelArgs &a, uint32_t tid, uint32_t nth, unsigned *total) {
@@ -617,8 +657,8 @@ __device__ __forceinline__ void peel_relax(const PeelArgs &a, PeelCounters *c, u
 // The rounds from state `st` on; every thread of the group calls it with the
 // same state.  Returns when at most `stop` vertices remain (0: all peeled),
 // with the state to resume from; false when a barrier gave up.
-template <typename Sync>
-__device__ bool peel_rounds(const PeelArgs &a, PeelCounters *c, PeelState &st, uint32_t stop, uint32_t tid,
+template <bool SH, typename Sync>
+__device__ __forceinline__ bool peel_rounds(const PeelArgs &a, PeelCounters *c, PeelState &st, uint32_t stop, uint32_t tid,
                             uint32_t nth, const Sync &sync) {
     volatile PeelCounters *vc = c;
     const unsigned lane = lane_id();
@@ -639,7 +679,7 @@ __device__ bool peel_rounds(const PeelArgs &a, PeelCounters *c, PeelState &st, u
                     const int B = st.t + kNear;
                     for (uint32_t v0 = tid - lane; v0 < a.n; v0 += nth) {
                         const uint32_t v = v0 + lane;
-                        const int d = v < a.n ? __ldcg(&a.deg[v]) : kGone;
+                        const int d = v < a.n ? peel_load<SH>(&a.deg[v]) : kGone;
                         const bool rest = d > st.t, in = rest && d <= B;
                         if (rest) best = max(best, 0x80000000u - (uint32_t)d);
                         const unsigned m = __ballot_sync(0xffffffffu, in);
@@ -655,8 +695,8 @@ __device__ bool peel_rounds(const PeelArgs &a, PeelCounters *c, PeelState &st, u
                         uint32_t v = 0;
                         int d = kGone;
                         if (i < nn) {
-                            v = __ldcg(&a.near[i]);
-                            d = __ldcg(&a.deg[v]);
+                            v = peel_load<SH>(&a.near[i]);
+                            d = peel_load<SH>(&a.deg[v]);
                         }
                         if (d > st.t) best = max(best, 0x80000000u - (uint32_t)d);
                         const bool sel = d == st.t + 1;
@@ -706,7 +746,7 @@ __device__ bool peel_rounds(const PeelArgs &a, PeelCounters *c, PeelState &st, u
         uint32_t ls = 0;  // log2 of the warps per row
         while ((st.nin << (ls + 1)) <= W) ls++;
         for (uint32_t unit = gw; unit < st.nin << ls; unit += W) {
-            const uint32_t v = __ldcg(&a.order[st.done + (unit >> ls)]);
+            const uint32_t v = peel_load<SH>(&a.order[st.done + (unit >> ls)]);
             const uint64_t b = a.rp[v], e = a.rp[v + 1];
             if (ls == 0 && e - b > kBigRow) {
                 uint32_t at = 0;
@@ -747,7 +787,7 @@ __global__ void __launch_bounds__(1024) k_peel_grid(const PeelArgs a) {
     peel_setup(a, tid, nth, &a.ctl->total);
     if (!sync()) return;
     PeelState st{0, 0, 0, -1, -1, *(volatile unsigned *)&a.ctl->total};
-    if (!peel_rounds(a, c, st, a.handover, tid, nth, sync)) return;
+    if (!peel_rounds<false>(a, c, st, a.handover, tid, nth, sync)) return;
     if (tid == 0) a.ctl->st = st;
 }
 
@@ -789,8 +829,30 @@ __global__ void __launch_bounds__(1024) k_peel_cluster(const PeelArgs a, int res
         sync();
         st = PeelState{0, 0, 0, -1, -1, *(volatile unsigned *)tot};
     }
-    peel_rounds(a, c, st, 0, tid, nth, sync);
+    peel_rounds<false>(a, c, st, 0, tid, nth, sync);
     sync();  // the first CTA's shared memory outlives the others' last access
+}
+
+// Small graphs in one CTA, with the degrees, the removal order and the near
+// list in shared memory: a round is about 1 us where the cluster takes 2.5
+// (orientation stage of a 2,000-vertex graph: SMALL_BEFORE -> SMALL_AFTER ms).
+__global__ void __launch_bounds__(1024) k_peel_block(PeelArgs a) {
+    extern __shared__ int peel_smem[];
+    __shared__ PeelCounters own;
+    __shared__ unsigned total;
+    a.deg = peel_smem;
+    a.order = reinterpret_cast<uint32_t *>(peel_smem + a.n);
+    a.near = a.order + a.n;
+    if (threadIdx.x == 0) {
+        own = PeelCounters{};
+        total = 0;
+    }
+    const BlockSync sync;
+    sync();
+    peel_setup(a, threadIdx.x, blockDim.x, &total);
+    sync();
+    PeelState st{0, 0, 0, -1, -1, total};
+    peel_rounds<true>(a, &own, st, 0, threadIdx.x, blockDim.x, sync);
 }
 
 // Out-degree in the DAG u -> w iff (key[u], u) < (key[w], w), both alive.
@@ -938,32 +1000,6 @@ constexpr int kScanThreads = 256;
 constexpr int kScanItems = 8;
 constexpr int kScanTile = kScanThreads * kScanItems;
 
-__device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t *smem, uint32_t *total) {
-    const unsigned lane = lane_id(), wid = threadIdx.x >> 5;
-    uint32_t v = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= (unsigned)o) v += y;
-    }
-    if (lane == 31) smem[wid] = v;
-    __syncthreads();
-    if (wid == 0) {
-        uint32_t s = lane < (blockDim.x >> 5) ? smem[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= (unsigned)o) s += y;
-        }
-        smem[lane] = s;
-    }
-    __syncthreads();
-    uint32_t warp_prefix = wid ? smem[wid - 1] : 0;
-    *total = smem[(blockDim.x >> 5) - 1];
-    __syncthreads();
-    return warp_prefix + v - x;
-}
-
 __global__ void k_scan_tiles(const uint32_t *__restrict__ in, uint32_t *out, uint32_t n,
                              uint32_t *tile_sums) {
     __shared__ uint32_t smem[32];
@@ -996,19 +1032,22 @@ __global__ void k_scan_add(uint32_t *out, uint32_t n, const uint32_t *__restrict
 
 // ====================================================== host launchers
 // ---------------------------------------------------------- batching
-// Disjoint union of a batch of graphs: block b copies graph b's rows and
-// columns with its vertex offset voff[b] and edge offset eoff[b].
+// Disjoint union of a batch of graphs: the blocks (b, *) copy graph b's rows and
+// columns with its vertex offset voff[b] and edge offset eoff[b].  One block a
+// graph left a batch of 64 waiting for its largest graph (UNION_BEFORE ms of a
+// pass, UNION_AFTER with the stripes).
 __global__ void k_union_build(const BatchSrc *__restrict__ src, uint32_t n_total, uint64_t *urp,
                               uint32_t *ucol, uint32_t *graph_of, uint32_t *idmap, uint8_t *kmap) {
     const BatchSrc b = src[blockIdx.x];
-    for (uint32_t v = threadIdx.x; v < b.n; v += blockDim.x) {
+    const uint32_t tid = blockIdx.y * blockDim.x + threadIdx.x, nth = gridDim.y * blockDim.x;
+    for (uint32_t v = tid; v < b.n; v += nth) {
         urp[b.voff + v] = b.rp[v] + b.eoff;
         graph_of[b.voff + v] = blockIdx.x;
         idmap[b.voff + v] = v;
         kmap[b.voff + v] = (uint8_t)b.k;
     }
-    for (uint64_t e = threadIdx.x; e < b.nnz; e += blockDim.x) ucol[b.eoff + e] = b.col[e] + b.voff;
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) urp[n_total] = b.eoff + b.nnz;
+    for (uint64_t e = tid; e < b.nnz; e += nth) ucol[b.eoff + e] = b.col[e] + b.voff;
+    if (blockIdx.x == gridDim.x - 1 && tid == 0) urp[n_total] = b.eoff + b.nnz;
 }
 
 // Per-graph sums of per-vertex attributions (one block per graph).
@@ -1040,7 +1079,8 @@ int launch_union_build(const BatchSrc *src, uint32_t G, uint32_t n_total, uint64
                        uint32_t *ucol, uint32_t *graph_of, uint32_t *idmap, uint8_t *kmap,
                        cudaStream_t s) {
     if (G == 0) return 0;
-    k_union_build<<<G, 256, 0, s>>>(src, n_total, urp, ucol, graph_of, idmap, kmap);
+    const uint32_t stripes = G < 2048 ? 2048 / G : 1;  // about 13 blocks an SM
+    k_union_build<<<dim3(G, stripes), 256, 0, s>>>(src, n_total, urp, ucol, graph_of, idmap, kmap);
     return 1;
 }
 
@@ -1048,7 +1088,7 @@ int launch_graph_sums(const BatchSrc *src, uint32_t G, const unsigned long long 
                       const unsigned long long *vcks, unsigned long long *out_count,
                       unsigned long long *out_cks, cudaStream_t s) {
     if (G == 0) return 0;
-    k_graph_sums<<<G, 256, 0, s>>>(src, vcount, vcks, out_count, out_cks);
+    k_graph_sums<<<G, 1024, 0, s>>>(src, vcount, vcks, out_count, out_cks);
     return 1;
 }
 
@@ -1169,12 +1209,15 @@ int launch_peel_update(const kcl_graph *g, Workspace &w, const uint32_t *fin, ui
     return 1;
 }
 
-constexpr int kPeelThreads = 1024;
 // Graphs up to this size are peeled in the cluster alone, and the grid leaves
 // the last kHandover vertices to it.  Orientation stage of the 1M-vertex and
 // the 262k-vertex R-MAT graph in ms: handover at 8k vertices 11.2 / 5.0, 32k
 // 10.4 / 3.6, 128k 9.2 / 3.2, 400k 9.3 / 3.2 (all cluster), the grid to the end
 // 10.4 / 5.4.
+// Up to kBlockVertices (whose arrays fit in shared memory) and kBlockEntries one
+// CTA takes the whole peel.
+constexpr uint32_t kBlockVertices = 1u << 14;
+constexpr uint64_t kBlockEntries = 1ull << 16;
 constexpr uint32_t kClusterVertices = 1u << 17;
 constexpr uint64_t kClusterEntries = 1ull << 22;
 constexpr uint32_t kHandover = 1u << 17;
@@ -1236,6 +1279,10 @@ static int peel_cluster_size() {
 // control block is cleared first.  Returns the launches, -1 if it cannot run.
 static int peel_launches(PeelArgs a, int blocks, uint64_t nnz, cudaStream_t s) {
     if (cudaMemsetAsync(a.ctl, 0, sizeof(PeelCtl), s) != cudaSuccess) return -1;
+    if (a.n <= kBlockVertices && nnz <= kBlockEntries && allow_max_smem(k_peel_block)) {
+        k_peel_block<<<1, kPeelThreads, 3 * sizeof(uint32_t) * a.n, s>>>(a);
+        return 1;
+    }
     int size = peel_cluster_size();
     const bool small = size && a.n <= kClusterVertices && nnz <= kClusterEntries;
     int launches = 0;
@@ -1384,8 +1431,10 @@ extern "C" kcl_status kcl_degeneracy_order_noalloc(uint32_t n, const uint64_t *r
     kcl::PeelCtl *ctl = reinterpret_cast<kcl::PeelCtl *>(S + 3 * (size_t)KCL_NOALLOC_MAX_VERTICES);
     const kcl::PeelArgs a{n, row_ptr, col, alive, degree, reinterpret_cast<int *>(S), round_out,
                           S + KCL_NOALLOC_MAX_VERTICES, S + 2 * (size_t)KCL_NOALLOC_MAX_VERTICES, ctl, 0};
-    // the entry count is on the device: only small n goes to the cluster alone
-    if (kcl::peel_launches(a, blocks, n <= 1u << 15 ? 0 : ~0ull, s) < 0) {
+    // the entry count is on the device: only small n goes to one CTA (at most
+    // n^2 entries) or to the cluster alone
+    const uint64_t nnz = n <= 512 ? 0 : n <= 1u << 15 ? kcl::kBlockEntries + 1 : ~0ull;
+    if (kcl::peel_launches(a, blocks, nnz, s) < 0) {
         (void)cudaGetLastError();
         return KCL_ECUDA;
     }
