@@ -21,9 +21,9 @@
 //     once per (node, a) and a clique costs one SplitMix64 round (two when
 //     the root's own id is the largest) instead of k and a merge.
 // Listing kernels of the 1M-vertex R-MAT graph (16 edges a vertex), before and
-// now: k = 5 colour count 179.3 -> 42.2 ms, k = 4 colour listing 201.2 -> 101.8
-// ms (2.06e10 records, 3.2 TB/s of stores; the stores alone would take 49 ms at
-// the measured copy bandwidth).  Counting is bound by the ALU pipe, listing by
+// now: k = 5 colour count 179.3 -> 42.2 ms, k = 4 colour listing 201.2 -> 99.4
+// ms (2.06e10 records, 3.3 TB/s of stores; the stores alone would take 43 ms at
+// the 7.7 TB/s that a fill writes here, the hashes alone 83).  Counting is bound by the ALU pipe, listing by
 // issue slots around the hash round.  A kernel per k: with all of k = 3..6 in
 // one, 45.0 and 106.0 ms (registers, instruction cache).
 #include "kcl_internal.cuh"
@@ -572,11 +572,9 @@ __device__ __forceinline__ void list_rows(const uint32_t *M, uint32_t WP, uint32
             if (DIRECT && (bl >> 5) == t) mw &= (1u << (bl & 31)) - 1u;
             idw = cid[bl];
         }
-        unsigned rows = __ballot_sync(kFull, mw != 0);
+        const uint32_t nrow = min(32u, (bend - b0 + bstep - 1) / bstep);
 #pragma unroll 1
-        while (rows) {
-            const int j = __ffs(rows) - 1;
-            rows &= rows - 1;
+        for (uint32_t j = 0; j < nrow; j++) {
             const uint32_t m = __shfl_sync(kFull, mw, j), idb = __shfl_sync(kFull, idw, j);
             uint64_t hb = mix64(h ^ (uint64_t)idb);
             if (TAIL) hb = mix64(hb ^ (uint64_t)u);
