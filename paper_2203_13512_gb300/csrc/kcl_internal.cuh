@@ -87,8 +87,11 @@ struct BatchSrc {
     uint32_t pad;
 };
 
-// Workspace owned by a graph, grown on demand and reused across calls.
+// Workspace owned by a graph, grown on demand and reused across calls; its arrays
+// (all device pointers but the arena) are carved from one allocation.
 struct Workspace {
+    void *slab = nullptr;
+    size_t slab_bytes = 0;
     uint8_t *alive = nullptr;        // n
     uint8_t *alive_core = nullptr;   // n (copy after Pre-Core, for stage info)
     uint32_t *cdeg = nullptr;        // n: current degree in the alive subgraph
