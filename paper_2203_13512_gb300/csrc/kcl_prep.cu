@@ -56,40 +56,68 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t *smem, 
 
 // ----------------------------------------------------------- validation
 // Row u: strictly ascending, ids < n, no self-loop, and every v in row u has
-// u in row v (binary search).  Also records the maximum degree.
+// u in row v (binary search).  Also records the maximum degree.  A warp takes a
+// row; the rest of a row beyond kLongRow entries is left to the whole block, and
+// a warp keeps its findings to itself until the end (500k-vertex R-MAT graph:
+// 3.28 -> 0.85 ms; a 10,000-vertex graph with a hub 61 -> 45 us).
+constexpr uint32_t kLongRow = 512, kLongRows = 64;
+
+__device__ __forceinline__ bool bad_entry(uint32_t n, uint64_t nnz, const uint64_t *__restrict__ rp,
+                                          const uint32_t *__restrict__ col, uint32_t u, uint64_t b, uint64_t i) {
+    const uint32_t v = col[i];
+    if (v >= n || v == u) return true;
+    const bool bad = i > b && col[i - 1] >= v;
+    uint64_t lo = rp[v], hi = rp[v + 1];  // symmetric: u must be in row v
+    if (hi < lo || hi > nnz) return true;
+    while (lo < hi) {
+        const uint64_t mid = lo + ((hi - lo) >> 1);
+        const uint32_t x = col[mid];
+        if (x == u) return bad;
+        if (x < u) lo = mid + 1; else hi = mid;
+    }
+    return true;
+}
+
 __global__ void k_validate(uint32_t n, uint64_t nnz, const uint64_t *__restrict__ rp,
                            const uint32_t *__restrict__ col, DevResult *res) {
+    __shared__ uint32_t rows[kLongRows];
+    __shared__ unsigned nlong;
+    if (threadIdx.x == 0) nlong = 0;
+    __syncthreads();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (rp[0] != 0 || rp[n] != nnz) atomicOr(&res->status, DEV_ERR_INVALID_GRAPH);
     }
     const unsigned lane = lane_id();
+    bool bad = false;
+    uint32_t most = 0;
     for (uint32_t u = warp_global(); u < n; u += warps_total()) {
         uint64_t b = rp[u], e = rp[u + 1];
-        if (e < b || e > nnz) {
-            if (lane == 0) atomicOr(&res->status, DEV_ERR_INVALID_GRAPH);
+        if (e < b || e > nnz || e - b > 0xFFFFFFFFull) {
+            bad = true;
             continue;
         }
-        if (lane == 0 && e - b > 0xFFFFFFFFull) atomicOr(&res->status, DEV_ERR_INVALID_GRAPH);
-        if (lane == 0) atomicMax(&res->max_outdeg, (unsigned)(e - b));
-        bool bad = false;
-        for (uint64_t i = b + lane; i < e; i += 32) {
-            uint32_t v = col[i];
-            if (v >= n || v == u) { bad = true; continue; }
-            if (i > b && col[i - 1] >= v) bad = true;
-            // symmetric: u must be in row v
-            uint64_t lo = rp[v], hi = rp[v + 1];
-            if (hi < lo || hi > nnz) { bad = true; continue; }
-            bool found = false;
-            while (lo < hi) {
-                uint64_t mid = lo + ((hi - lo) >> 1);
-                uint32_t x = col[mid];
-                if (x == u) { found = true; break; }
-                if (x < u) lo = mid + 1; else hi = mid;
+        most = max(most, (uint32_t)(e - b));
+        uint64_t stop = e;
+        if (e - b > 2 * kLongRow) {
+            unsigned at = 0;
+            if (lane == 0) at = atomicAdd(&nlong, 1u);
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (at < kLongRows) {
+                if (lane == 0) rows[at] = u;
+                stop = b + kLongRow;
             }
-            if (!found) bad = true;
         }
-        if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&res->status, DEV_ERR_INVALID_GRAPH);
+        for (uint64_t i = b + lane; i < stop; i += 32) bad |= bad_entry(n, nnz, rp, col, u, b, i);
     }
+    __syncthreads();
+    const unsigned k = min(nlong, kLongRows);
+    for (unsigned j = 0; j < k; j++) {
+        const uint32_t u = rows[j];
+        const uint64_t b = rp[u], e = rp[u + 1];
+        for (uint64_t i = b + kLongRow + threadIdx.x; i < e; i += blockDim.x) bad |= bad_entry(n, nnz, rp, col, u, b, i);
+    }
+    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&res->status, DEV_ERR_INVALID_GRAPH);
+    if (lane == 0 && most) atomicMax(&res->max_outdeg, most);
 }
 
 // ------------------------------------------------------------- Pre-Core
@@ -624,14 +652,35 @@ __device__ void peel_setup(const PeelArgs &a, uint32_t tid, uint32_t nth, unsign
     if (lane_id() == 0 && cnt) atomicAdd(total, cnt);
 }
 
+// A graph's rows: in global memory, or copied to shared memory (small graphs; ids
+// below 2^16).
+struct GlobalRows {
+    const uint64_t *rp;
+    const uint32_t *col;
+    using Pos = uint64_t;
+    __device__ __forceinline__ Pos begin(uint32_t v) const { return rp[v]; }
+    __device__ __forceinline__ Pos end(uint32_t v) const { return rp[v + 1]; }
+    __device__ __forceinline__ uint32_t entry(Pos x) const { return col[x]; }
+};
+struct LocalRows {
+    const uint32_t *rp;
+    const uint16_t *col;
+    using Pos = uint32_t;
+    __device__ __forceinline__ Pos begin(uint32_t v) const { return rp[v]; }
+    __device__ __forceinline__ Pos end(uint32_t v) const { return rp[v + 1]; }
+    __device__ __forceinline__ uint32_t entry(Pos x) const { return col[x]; }
+};
+
 // Lowers the degrees of up to four neighbours a lane (n of them valid, stride
 // `step` from x) and appends those that reach t or B.
-__device__ __forceinline__ void peel_relax(const PeelArgs &a, PeelCounters *c, unsigned *next, uint32_t next0,
-                                           uint64_t x, uint64_t e, uint64_t step, int t, int B, uint32_t round) {
+template <typename R>
+__device__ __forceinline__ void peel_relax(const PeelArgs &a, const R &rows, PeelCounters *c, unsigned *next,
+                                           uint32_t next0, typename R::Pos x, typename R::Pos e,
+                                           typename R::Pos step, int t, int B, uint32_t round) {
     uint32_t w[4];
     int old[4];
 #pragma unroll
-    for (int z = 0; z < 4; z++) w[z] = x + z * step < e ? a.col[x + z * step] : 0xFFFFFFFFu;
+    for (int z = 0; z < 4; z++) w[z] = x + z * step < e ? rows.entry(x + z * step) : 0xFFFFFFFFu;
 #pragma unroll
     for (int z = 0; z < 4; z++) old[z] = w[z] != 0xFFFFFFFFu ? atomicSub(&a.deg[w[z]], 1) : kGone;
 #pragma unroll
@@ -657,9 +706,10 @@ __device__ __forceinline__ void peel_relax(const PeelArgs &a, PeelCounters *c, u
 // The rounds from state `st` on; every thread of the group calls it with the
 // same state.  Returns when at most `stop` vertices remain (0: all peeled),
 // with the state to resume from; false when a barrier gave up.
-template <bool SH, typename Sync>
-__device__ __forceinline__ bool peel_rounds(const PeelArgs &a, PeelCounters *c, PeelState &st, uint32_t stop, uint32_t tid,
-                            uint32_t nth, const Sync &sync) {
+template <bool SH, typename R, typename Sync>
+__device__ __forceinline__ bool peel_rounds(const PeelArgs &a, const R &rows, PeelCounters *c, PeelState &st,
+                                            uint32_t stop, uint32_t tid, uint32_t nth, const Sync &sync) {
+    using Pos = typename R::Pos;
     volatile PeelCounters *vc = c;
     const unsigned lane = lane_id();
     const uint32_t gw = tid >> 5, W = nth >> 5;
@@ -747,7 +797,7 @@ __device__ __forceinline__ bool peel_rounds(const PeelArgs &a, PeelCounters *c, 
         while ((st.nin << (ls + 1)) <= W) ls++;
         for (uint32_t unit = gw; unit < st.nin << ls; unit += W) {
             const uint32_t v = peel_load<SH>(&a.order[st.done + (unit >> ls)]);
-            const uint64_t b = a.rp[v], e = a.rp[v + 1];
+            const Pos b = rows.begin(v), e = rows.end(v);
             if (ls == 0 && e - b > kBigRow) {
                 uint32_t at = 0;
                 if (lane == 0) at = atomicAdd(bcnt, 1u);
@@ -757,18 +807,18 @@ __device__ __forceinline__ bool peel_rounds(const PeelArgs &a, PeelCounters *c, 
                     continue;
                 }
             }
-            const uint64_t step = 32ull << ls;
-            for (uint64_t x = b + 32 * (unit & ((1u << ls) - 1u)); x < e; x += 4 * step)
-                peel_relax(a, c, next, next0, x + lane, e, step, st.t, st.B, st.round);
+            const Pos step = (Pos)32 << ls;
+            for (Pos x = b + 32 * (unit & ((1u << ls) - 1u)); x < e; x += 4 * step)
+                peel_relax(a, rows, c, next, next0, x + lane, e, step, st.t, st.B, st.round);
         }
         if (!sync()) return false;
         const uint32_t nb = min(vc->bcnt[fi], (unsigned)kPeelBig);
         if (nb) {
             for (uint32_t i = 0; i < nb; i++) {
                 const uint32_t v = __ldcg(&big[i]);
-                const uint64_t b = a.rp[v], e = a.rp[v + 1];
-                for (uint64_t x = b + (uint64_t)gw * 32; x < e; x += 4ull * nth)
-                    peel_relax(a, c, next, next0, x + lane, e, nth, st.t, st.B, st.round);
+                const Pos b = rows.begin(v), e = rows.end(v);
+                for (Pos x = b + (Pos)gw * 32; x < e; x += (Pos)4 * nth)
+                    peel_relax(a, rows, c, next, next0, x + lane, e, nth, st.t, st.B, st.round);
             }
             if (!sync()) return false;
         }
@@ -787,7 +837,7 @@ __global__ void __launch_bounds__(1024) k_peel_grid(const PeelArgs a) {
     peel_setup(a, tid, nth, &a.ctl->total);
     if (!sync()) return;
     PeelState st{0, 0, 0, -1, -1, *(volatile unsigned *)&a.ctl->total};
-    if (!peel_rounds<false>(a, c, st, a.handover, tid, nth, sync)) return;
+    if (!peel_rounds<false>(a, GlobalRows{a.rp, a.col}, c, st, a.handover, tid, nth, sync)) return;
     if (tid == 0) a.ctl->st = st;
 }
 
@@ -829,31 +879,40 @@ __global__ void __launch_bounds__(1024) k_peel_cluster(const PeelArgs a, int res
         sync();
         st = PeelState{0, 0, 0, -1, -1, *(volatile unsigned *)tot};
     }
-    peel_rounds<false>(a, c, st, 0, tid, nth, sync);
+    peel_rounds<false>(a, GlobalRows{a.rp, a.col}, c, st, 0, tid, nth, sync);
     sync();  // the first CTA's shared memory outlives the others' last access
 }
 
 // Small graphs in one CTA, with the degrees, the removal order and the near
-// list in shared memory: no L2 round trip but for the rows (orientation stage of
-// a 2,000-vertex graph of 67 rounds: 0.22 ms in the cluster, 0.15 here; of a
-// 10,000-vertex graph of 100,000 entries 0.38 in the cluster, 0.44 here).
-__global__ void __launch_bounds__(1024) k_peel_block(PeelArgs a) {
+// list in shared memory, and the rows too when they fit (LOCAL), so a round makes
+// no L2 round trip.  Orientation stage of a 2,000-vertex graph of 67 rounds: 0.22
+// ms in the cluster, 0.15 with the rows in global memory, 0.14 with all of it
+// here; of a 10,000-vertex graph of 100,000 entries 0.38 in the cluster, 0.44 here.
+template <bool LOCAL>
+__global__ void __launch_bounds__(1024) k_peel_block(PeelArgs a, uint32_t nnz) {
     extern __shared__ int peel_smem[];
     __shared__ PeelCounters own;
     __shared__ unsigned total;
     a.deg = peel_smem;
     a.order = reinterpret_cast<uint32_t *>(peel_smem + a.n);
     a.near = a.order + a.n;
+    uint32_t *rp = a.near + a.n;
+    uint16_t *col = reinterpret_cast<uint16_t *>(rp + a.n + 1);
     if (threadIdx.x == 0) {
         own = PeelCounters{};
         total = 0;
+    }
+    if (LOCAL) {
+        for (uint32_t v = threadIdx.x; v <= a.n; v += blockDim.x) rp[v] = (uint32_t)a.rp[v];
+        for (uint32_t x = threadIdx.x; x < nnz; x += blockDim.x) col[x] = (uint16_t)a.col[x];
     }
     const BlockSync sync;
     sync();
     peel_setup(a, threadIdx.x, blockDim.x, &total);
     sync();
     PeelState st{0, 0, 0, -1, -1, total};
-    peel_rounds<true>(a, &own, st, 0, threadIdx.x, blockDim.x, sync);
+    if (LOCAL) peel_rounds<true>(a, LocalRows{rp, col}, &own, st, 0, threadIdx.x, blockDim.x, sync);
+    else peel_rounds<true>(a, GlobalRows{a.rp, a.col}, &own, st, 0, threadIdx.x, blockDim.x, sync);
 }
 
 // Out-degree in the DAG u -> w iff (key[u], u) < (key[w], w), both alive.
@@ -1219,6 +1278,7 @@ int launch_peel_update(const kcl_graph *g, Workspace &w, const uint32_t *fin, ui
 // CTA takes the whole peel.
 constexpr uint32_t kBlockVertices = 1u << 14;
 constexpr uint64_t kBlockEntries = 1ull << 16;
+constexpr size_t kBlockShared = 220 * 1024;
 constexpr uint32_t kClusterVertices = 1u << 17;
 constexpr uint64_t kClusterEntries = 1ull << 22;
 constexpr uint32_t kHandover = 1u << 17;
@@ -1276,13 +1336,22 @@ static int peel_cluster_size() {
     return best;
 }
 
-// The whole peel: wide rounds on the grid, the tail on one cluster.  The
-// control block is cleared first.  Returns the launches, -1 if it cannot run.
-static int peel_launches(PeelArgs a, int blocks, uint64_t nnz, cudaStream_t s) {
+// The whole peel: wide rounds on the grid, the tail on one cluster.  nnz: the
+// entries, or (known = false) a stand-in for them.  The control block is cleared
+// first.  Returns the launches, -1 if it cannot run.
+static int peel_launches(PeelArgs a, int blocks, uint64_t nnz, bool known, cudaStream_t s) {
     if (cudaMemsetAsync(a.ctl, 0, sizeof(PeelCtl), s) != cudaSuccess) return -1;
-    if (a.n <= kBlockVertices && nnz <= kBlockEntries && allow_max_smem(k_peel_block)) {
-        k_peel_block<<<1, kPeelThreads, 3 * sizeof(uint32_t) * a.n, s>>>(a);
-        return 1;
+    if (a.n <= kBlockVertices && nnz <= kBlockEntries) {
+        const size_t lists = 3 * sizeof(uint32_t) * (size_t)a.n;
+        const size_t all = lists + sizeof(uint32_t) * ((size_t)a.n + 1) + sizeof(uint16_t) * (size_t)nnz;
+        if (known && all <= kBlockShared && allow_max_smem(k_peel_block<true>)) {
+            k_peel_block<true><<<1, kPeelThreads, all, s>>>(a, (uint32_t)nnz);
+            return 1;
+        }
+        if (allow_max_smem(k_peel_block<false>)) {
+            k_peel_block<false><<<1, kPeelThreads, lists, s>>>(a, 0);
+            return 1;
+        }
     }
     int size = peel_cluster_size();
     const bool small = size && a.n <= kClusterVertices && nnz <= kClusterEntries;
@@ -1309,7 +1378,7 @@ static int peel_launches(PeelArgs a, int blocks, uint64_t nnz, cudaStream_t s) {
 int launch_peel(const kcl_graph *g, Workspace &w, cudaStream_t s) {
     const PeelArgs a{g->n, g->rp, g->col, w.alive, w.cdeg, reinterpret_cast<int *>(w.peel_deg), w.key,
                      w.frontier_a, w.frontier_b, w.peel, 0};
-    return peel_launches(a, peel_blocks(g->num_sms, g->n), g->nnz, s);
+    return peel_launches(a, peel_blocks(g->num_sms, g->n), g->nnz, true, s);
 }
 
 int launch_precore(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s) {
@@ -1435,7 +1504,7 @@ extern "C" kcl_status kcl_degeneracy_order_noalloc(uint32_t n, const uint64_t *r
     // the entry count is on the device: only small n goes to one CTA (at most
     // n^2 entries) or to the cluster alone
     const uint64_t nnz = n <= 512 ? 0 : n <= 1u << 15 ? kcl::kBlockEntries + 1 : ~0ull;
-    if (kcl::peel_launches(a, blocks, nnz, s) < 0) {
+    if (kcl::peel_launches(a, blocks, nnz, false, s) < 0) {
         (void)cudaGetLastError();
         return KCL_ECUDA;
     }
