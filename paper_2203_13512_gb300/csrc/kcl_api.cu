@@ -104,10 +104,12 @@ void mirror_give(DevResult *p) {
     else cudaFreeHost(p);
 }
 
-// Everything but the arena is one allocation (w.slab).
+// Everything but a large arena is one allocation (w.slab).
+constexpr size_t kSmallArena = 1024;  // words
+
 void free_workspace(Workspace &w) {
+    if (w.arena && w.arena != w.small_arena) cudaFree(w.arena);
     if (w.slab) cudaFree(w.slab);
-    if (w.arena) cudaFree(w.arena);
     mirror_give(w.h_res);
     w = Workspace();
 }
@@ -126,9 +128,10 @@ kcl_status ensure_workspace(kcl_graph *g) {
         n_new = (uint32_t)std::min<uint64_t>(0xFFFFFFF0ull, std::max<uint64_t>(g->n, w.n_cap + w.n_cap / 2));
         nnz_new = std::max<uint64_t>(g->nnz, w.nnz_cap + w.nnz_cap / 2);
     }
-    size_t arena_words = w.arena_words;
-    uint32_t *arena = w.arena;
-    w.arena = nullptr;
+    const bool own_arena = w.arena && w.arena != w.small_arena;
+    const size_t arena_words = own_arena ? w.arena_words : 0;
+    uint32_t *arena = own_arena ? w.arena : nullptr;
+    if (own_arena) w.arena = nullptr;
     if (w.h_res) KCL_CK(cudaStreamSynchronize(g->stream));  // the mirror goes back to the pool
     free_workspace(w);
     w.arena = arena;  // the arena is sized separately (ensure_arena)
@@ -147,6 +150,7 @@ kcl_status ensure_workspace(kcl_graph *g) {
         carve(&w.peel, 1);
         carve(&w.queue, 64);
         carve(&w.slots, kMaxSplitSlots);
+        carve(&w.small_arena, kSmallArena);
         carve(&w.alive, n);
         carve(&w.alive_core, n);
         carve(&w.cdeg, n);
@@ -187,9 +191,18 @@ kcl_status ensure_workspace(kcl_graph *g) {
     return KCL_OK;
 }
 
+// At least `words` of arena; a few words come out of the workspace, so calls
+// that need (almost) none allocate nothing.
 kcl_status ensure_arena(kcl_graph *g, size_t words) {
     Workspace &w = g->ws;
+    if (w.arena_words == 0 && words <= kSmallArena) {
+        w.arena = w.small_arena;
+        w.arena_words = kSmallArena;
+        return KCL_OK;
+    }
     if (words <= w.arena_words) return KCL_OK;
+    if (w.arena == w.small_arena) w.arena = nullptr;
+    w.arena_words = 0;
     KCL_TRY(dev_alloc(&w.arena, words));
     w.arena_words = words;
     return KCL_OK;
@@ -429,10 +442,13 @@ kcl_status run_call(kcl_graph *g, uint32_t k, kcl_ordering ord, const kcl_ring *
     if (fe.n_roots > 0 && g->time_limit_ms)
         T.add(3, launch_set_deadline(w.res, g->time_limit_ms, g->stream));
     if (fe.n_roots > 0) {
-        size_t arena = ord == KCL_ORDER_DEGREE
-                           ? sdegree_arena_words(k, g->num_sms, fe.max_outdeg)
-                           : bitcol_arena_words(k, g->num_sms, fe.max_outdeg);
-        if (k <= 6) arena = std::max(arena, sub_arena_words(g->num_sms, fe.max_outdeg, listing));
+        // the classes of the id-ordered kernels need only their own
+        bool sub = fe.max_outdeg <= kSubMaxOutdeg;
+        for (int c = 0; c < fe.n_classes && fe.limits[c] <= kSubMaxOutdeg; c++) sub = sub && sub_handles(g, k, c, ord);
+        size_t arena = k <= 6 ? sub_arena_words(k, g->num_sms, fe.max_outdeg, listing) : 0;
+        if (!sub)
+            arena = std::max(arena, ord == KCL_ORDER_DEGREE ? sdegree_arena_words(k, g->num_sms, fe.max_outdeg)
+                                                            : bitcol_arena_words(k, g->num_sms, fe.max_outdeg));
         KCL_TRY(ensure_arena(g, arena));
         int l = ord == KCL_ORDER_DEGREE
                     ? launch_sdegree(g, k, w, fe.class_begin, fe.n_classes, la, g->stream)

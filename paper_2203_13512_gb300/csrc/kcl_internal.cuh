@@ -113,6 +113,7 @@ struct Workspace {
     uint32_t *members = nullptr;     // n: clique-component members (listing)
     uint32_t *comp_slot = nullptr;   // n: clique-component slot (listing)
     uint32_t *arena = nullptr;       // global scratch for large subproblems
+    uint32_t *small_arena = nullptr; // the arena of calls that need almost none
     unsigned long long *slots = nullptr;  // work-splitting slots, one per CTA of a launch
     size_t arena_words = 0;
     DevResult *res = nullptr;
@@ -589,8 +590,9 @@ int launch_bitcol(const kcl_graph *g, uint32_t k, Workspace &w, const uint32_t *
 
 // kcl_sub.cu: id-ordered subproblems (k <= 6, d+ <= 1024), both orderings.
 // sub_handles: whether class c of a call (k: the largest of a batch) runs there.
+constexpr uint32_t kSubMaxOutdeg = 1024;
 bool sub_handles(const kcl_graph *g, uint32_t k, int c, kcl_ordering ord);
-size_t sub_arena_words(int num_sms, uint32_t max_outdeg, bool listing);
+size_t sub_arena_words(uint32_t k, int num_sms, uint32_t max_outdeg, bool listing);
 int launch_sub(const kcl_graph *g, uint32_t k, Workspace &w, int c, uint32_t begin, uint32_t end, unsigned *queue,
                const ListArgs &la, uint32_t dfs_warps, cudaStream_t s);
 

@@ -698,9 +698,15 @@ __device__ void list_node(const uint32_t *A, uint32_t WP, const uint32_t *C, uin
 }
 
 // ------------------------------------------------------------------ walk
+// Where paths are two and more vertices long (k = 6 counting, k >= 5 listing) a
+// first-level child is a big unit: in the classes of few, large roots its own
+// children are dealt out in kSlices shares (d+ 257..354 of the 131k-vertex R-MAT
+// graph at k = 6: 16.0 -> 12.7 ms; in the smaller classes it cost 4 to 16 %).
+constexpr uint32_t kSlices = 4;
 struct Sub {
     const uint32_t *A, *nbr;
     uint32_t WP, W, d, u, ru;
+    uint32_t slice, slices;  // the share of a first-level child's own children this walk takes
     unsigned long long deadline;
 };
 
@@ -743,11 +749,13 @@ __device__ void walk(const Sub &s, uint32_t last, uint32_t c, uint32_t *path, co
         cnt += tri_count(s.A, s.WP, C, nw, c, sc);
     } else {
         uint32_t *Cn = sc.cb + J * s.W;
+        uint32_t at = 0;
         for (uint32_t t = w0; t < nw; t++) {
             uint32_t m = C[t];
             while (m) {
                 const uint32_t w = t * 32 + (__ffs(m) - 1);
                 m &= m - 1;
+                if (J == 1 && at++ % s.slices != s.slice) continue;
                 const uint32_t n = next_set<LIST>(s, C, w, Cn);
                 if (n + J + 2 >= K) {  // K - J - 2 more vertices needed
                     if (LIST) path[J] = s.nbr[w];
@@ -842,7 +850,7 @@ __device__ __forceinline__ void run(const SubArgs &a) {
         if (!skip) {
             const Rows rows = LIST ? kBoth : k > 3 ? kLower : kNoRows;
             const uint32_t hits = build<CTA>(d, base, a, L, S, rows);
-            Sub s{S + L.A, S + L.NBR, L.WP, L.W, d, u, 0u, deadline};
+            Sub s{S + L.A, S + L.NBR, L.WP, L.W, d, u, 0u, 0u, 1u, deadline};
             if (LIST) {
                 uint32_t below = 0;  // members with an id below u
                 for (uint32_t i = lane; i < d; i += 32) below += s.nbr[i] < u ? 1u : 0u;
@@ -860,14 +868,16 @@ __device__ __forceinline__ void run(const SubArgs &a) {
             } else if (G::warp() < nd) {
                 // the part's children, the ones with the most candidates first
                 const uint32_t nch = part < d ? (d - 1 - part) / a.parts + 1 : 0u;
+                if (CTA && a.D > 256 && (LIST ? k > 4 : k > 5)) s.slices = kSlices;
                 uint32_t i = 0;
                 for (;; i++) {
                     if (CTA) {
                         if (lane == 0) i = atomicAdd(&meta[1], 1u);
                         i = __shfl_sync(kFull, i, 0);
                     }
-                    if (i >= nch || warp_past_deadline(deadline, a.res)) break;
-                    const uint32_t v = LIST ? part + i * a.parts : d - 1 - part - i * a.parts;
+                    if (i >= nch * s.slices || warp_past_deadline(deadline, a.res)) break;
+                    const uint32_t v = LIST ? part + i / s.slices * a.parts : d - 1 - part - i / s.slices * a.parts;
+                    s.slice = i % s.slices;
                     if (k == 4) child<4, LIST>(s, v, sc, a, cnt, cks);
                     else if (k == 5) child<5, LIST>(s, v, sc, a, cnt, cks);
                     else child<6, LIST>(s, v, sc, a, cnt, cks);
@@ -910,13 +920,22 @@ struct Cfg {
     uint32_t per_sm;  // CTAs per SM the global room is sized for
 };
 
+// Whether class c runs a CTA per root.  Listing hashes every clique, and at k = 6
+// a root's cost grows with the square of its near-cliques: one warp on the
+// heaviest root then outlasts the launch (d+ 65..128 of the 131k-vertex R-MAT
+// graph: a warp per root 19.6 ms, a CTA 3.7; d+ 33..64 2.1 and 0.75).  Up to k =
+// 5 the warp form is the faster one up to d+ = 128 (3.5 against 3.6 ms on 1M
+// vertices), and up to d+ = 32 always (the community graph's 292,000 roots at k =
+// 6: 0.9 against 1.5 ms).
+bool cta_form(int c, uint32_t k, bool listing) { return listing || c >= kWarpClasses || (k > 5 && c > 0); }
+
 // Launch shape of class c for a largest out-degree maxd.
-Cfg config(int c, uint32_t maxd, bool listing) {
+Cfg config(int c, uint32_t k, uint32_t maxd, bool listing) {
     Cfg f;
     uint32_t d = maxd < kLimits[c] ? maxd : kLimits[c];
     f.D = (d + 31) & ~31u;
     if (f.D < 32) f.D = 32;
-    const bool cta = listing || c >= kWarpClasses;
+    const bool cta = cta_form(c, k, listing);
     const uint32_t full = set_room(f.D, listing);
     const uint32_t least = idx_words(f.D), fixed = scratch_fixed(row_words4(f.D));
     if (!cta) {
@@ -955,11 +974,11 @@ bool sub_handles(const kcl_graph *g, uint32_t k, int c, kcl_ordering ord) {
     return !(g->options & KCL_OPT_NO_COLOR_PRUNE);  // the ablation runs the colour path without its prune
 }
 
-size_t sub_arena_words(int num_sms, uint32_t max_outdeg, bool listing) {
+size_t sub_arena_words(uint32_t k, int num_sms, uint32_t max_outdeg, bool listing) {
     size_t need = 0;
     for (int c = 0; c < kSubClasses; c++) {
         if (c > 0 && kLimits[c - 1] >= max_outdeg) break;
-        const Cfg f = config(c, max_outdeg, listing);
+        const Cfg f = config(c, k, max_outdeg, listing);
         const size_t words = (size_t)f.gwords * f.warps * f.per_sm * (size_t)num_sms;
         if (words > need) need = words;
     }
@@ -968,7 +987,7 @@ size_t sub_arena_words(int num_sms, uint32_t max_outdeg, bool listing) {
 
 int launch_sub(const kcl_graph *g, uint32_t k, Workspace &w, int c, uint32_t begin, uint32_t end, unsigned *queue,
                const ListArgs &la, uint32_t dfs_warps, cudaStream_t s) {
-    const Cfg f = config(c, la.max_outdeg, la.listing);
+    const Cfg f = config(c, k, la.max_outdeg, la.listing);
     SubArgs a;
     a.optr = w.optr;
     a.oadj = w.oadj;
@@ -990,7 +1009,7 @@ int launch_sub(const kcl_graph *g, uint32_t k, Workspace &w, int c, uint32_t beg
     a.per_root = la.per_root;
     a.root_cks = la.per_root_cks;
     a.res = w.res;
-    const bool cta = la.listing || c >= kWarpClasses;
+    const bool cta = cta_form(c, k, la.listing);
     int occ = 0;
     uint32_t n = end - begin;
     using Kernel = void (*)(const SubArgs);
@@ -1017,9 +1036,10 @@ int launch_sub(const kcl_graph *g, uint32_t k, Workspace &w, int c, uint32_t beg
     if (occ < 1) occ = 1;
     if (occ > (int)f.per_sm) occ = (int)f.per_sm;  // global room per SM
     uint32_t blocks = (uint32_t)g->num_sms * occ;
-    // a class with few roots shares each root's children over several CTAs,
-    // which all build it
-    if (c >= kWarpClasses && (k >= 5 || (la.listing && k >= 4))) {
+    // a class with few roots shares each root's children over several CTAs, which
+    // all build it: up to 8 units per CTA of the launch (with up to 32, building
+    // took over: 131k k = 6 count 41.7 -> 60.6 ms; with up to 4, the tail: 43.1)
+    if (k >= 5 || (la.listing && k >= 4 && c >= kWarpClasses)) {
         while (a.parts < 8 && n * a.parts < 8 * blocks) a.parts *= 2;
     }
     if (blocks > n * a.parts) blocks = n * a.parts;
