@@ -415,7 +415,9 @@ def roofline(per_call, steps, peaks, sm_mhz, modes=("count", "list")):
         measured round rate / k.
     `achieved` = the oracle's count of that unit for the roots of that class
     (tests/golden/rmat20_work.json, split by out-degree) / that launch's
-    CUDA-event time."""
+    CUDA-event time.  The units are the paper's: the id-ordered kernels close
+    the same cliques with fewer words (compacted candidate sets) and fewer
+    rounds (shared chains), so a fraction may exceed 1."""
     work = _load_work()
     fam = {}
     for (k, o, m, c, ms, la, cl) in per_call:
@@ -489,45 +491,21 @@ def frontend_roofline(per_call, steps, n, nnz):
     return out
 
 
-# listing kernels of the out-degree classes (count mode), by (ordering, mode,
-# class index); classes as in kcl_sdegree.cu / kcl_bitcol.cu
+# listing kernels of the step's calls (k = 4, 5), by (ordering, mode, class
+# index): both orderings run the id-ordered kernels of kcl_sub.cu, a warp per
+# root up to d+ = 128 when counting, else a CTA per root
 KERNEL_NAMES = {
-    ("degree", "count", 0): "k_sdegree<0,0,1> (warp per root, d+ <= 32)",
-    ("degree", "count", 1): "k_sdegree<0,0,1> (warp per root, d+ <= 64)",
-    ("degree", "count", 2): "k_sdegree<0,0,1> (warp per root, d+ <= 128)",
-    ("degree", "count", 3): "k_sdegree_cta<0> (CTA per root, d+ <= 256)",
-    ("degree", "count", 4): "k_sdegree_cta<0> (CTA per root, d+ <= 512)",
-    ("degree", "count", 5): "k_sdegree_cta<0> (CTA per root, d+ <= 1024)",
-    ("color", "count", 0): "k_bitcol_warp<1,0>",
-    ("color", "count", 1): "k_bitcol_warp<2,0>",
-    ("color", "count", 2): "k_bitcol_warp<4,0>",
-    ("color", "count", 3): "k_bitcol_cta<8,0,0,0>",
-    ("color", "count", 4): "k_bitcol_cta<16,0,0,0>",
-    ("color", "count", 5): "k_bitcol_cta<16,0,1,0>",
-    ("degree", "list", 0): "k_sdegree_cta<1> (d+ <= 32)",
-    ("degree", "list", 1): "k_sdegree_cta<1> (d+ <= 64)",
-    ("degree", "list", 2): "k_sdegree_cta<1> (d+ <= 128)",
-    ("degree", "list", 3): "k_sdegree_cta<1> (d+ <= 256)",
-    ("degree", "list", 4): "k_sdegree_cta<1> (d+ <= 512)",
-    ("degree", "list", 5): "k_sdegree_cta<1> (d+ <= 1024)",
-    ("color", "list", 0): "k_bitcol_cta<4,1,0,0> (W=1)",
-    ("color", "list", 1): "k_bitcol_cta<4,1,0,0> (W=2)",
-    ("color", "list", 2): "k_bitcol_cta<4,1,0,0> (W=4)",
-    ("color", "list", 3): "k_bitcol_cta<8,1,0,0>",
-    ("color", "list", 4): "k_bitcol_cta<16,1,0,0>",
-    ("color", "list", 5): "k_bitcol_cta<16,1,1,0>",
+    (o, m, c): "%s (d+ <= %d)" % ("k_sub_warp<k>" if m == "count" and c < 3
+                                  else "k_sub_cta<%d, k>" % (m == "list"), lim)
+    for o in ("degree", "color") for m in ("count", "list")
+    for c, lim in enumerate((32, 64, 128, 256, 512, 1024))
 }
 
 # DRAM bytes (read + write) per launch of the listing launches from one ncu
 # capture of the same workload, keyed (k, ordering, mode, class); the source
 # names the summary under profiles/.  An entry is removed when its kernel
 # changes, until a new capture exists.
-_DRAM = "profiles/k_bitcol_cta_rmat20.md"
-TRAFFIC = {
-    (5, "color", "count", 4): (30.719e6 + 0.040e6, _DRAM),
-    (4, "color", "list", 4): (3.352e9 + 192.248e9, _DRAM),
-    (4, "degree", "list", 4): (6.684e9 + 190.315e9, "profiles/k_sdegree_cta_rmat20.md"),
-}
+TRAFFIC = {}
 
 
 def class_work(entry, lo, hi, field="work_by_outdeg"):

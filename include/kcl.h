@@ -64,7 +64,12 @@ typedef enum {
  *   the degeneracy DAG (bulk peel rounds: eta = (round, id)), then for each
  *   root the subgraph induced by its out-neighbours, greedy colour ordering
  *   (Section VII-A), bitmap encoding (Section VII-C) and BitColList with
- *   colour pruning. */
+ *   colour pruning.
+ * For k <= 6 and root out-degrees up to 1024 both orderings keep their DAG but
+ * orient the subgraph inside a root's out-neighbours by vertex id (any acyclic
+ * orientation finds each clique once): no colouring, ranks or lists.  SDegree's
+ * lists (kcl_tuning.sdegree_bitmap = 0xFFFFFFFF) and the colour-prune ablation
+ * (KCL_OPT_NO_COLOR_PRUNE) select the kernels of the algorithms as written. */
 typedef enum { KCL_ORDER_DEGREE = 0, KCL_ORDER_COLOR = 1 } kcl_ordering;
 
 /* Largest supported k (the paper requires k >= 3, Section III-A). */
@@ -292,9 +297,10 @@ kcl_status kcl_set_options(kcl_graph *g, uint32_t flags);
 kcl_status kcl_get_options(const kcl_graph *g, uint32_t *flags);
 
 /* Device scratch the graph handle holds now (Section IX's memory study): the
- * per-call workspace (about 74 bytes per vertex and 2 per CSR entry, grown to
- * the largest graph seen) and the listing arena (shared-memory spill of the
- * largest subproblems, sized by k and the largest out-degree), in bytes.
+ * per-call workspace (one allocation of about 74 bytes per vertex and 2 per CSR
+ * entry, grown to the largest graph seen) and the listing arena (shared-memory
+ * spill of the largest subproblems, sized by k and the largest out-degree; the
+ * few words a small graph needs lie in the workspace), in bytes.
  * The input CSR itself (8 (n+1) + 4 nnz bytes) is not included. */
 kcl_status kcl_scratch_bytes(const kcl_graph *g, uint64_t *workspace, uint64_t *arena);
 
@@ -326,6 +332,8 @@ kcl_status kcl_scratch_bytes(const kcl_graph *g, uint64_t *workspace, uint64_t *
  *   runs out of roots rebuilds the subproblem of a root still in progress on
  *   another CTA and takes over some of its children when at least t =
  *   split[c] of them are left; 0 = off (default).
+ * The id-ordered kernels (k <= 6, see the orderings above) use cta_warps only;
+ * they share heavy roots between CTAs by a rule of their own.
  * A graph starts with the defaults; views and batches start with the
  * defaults too. */
 typedef struct {
@@ -358,8 +366,8 @@ kcl_status kcl_autotune(kcl_graph *g, uint32_t k, kcl_ordering ord, int listing,
  * host program whose device memory is owned by another allocator under a
  * fixed budget.  This call computes the same bulk-peel rounds as the
  * KCL_ORDER_COLOR front end (eta = (round, id); see kcl_stage_info's `key`)
- * without allocating anything: its scratch (peel degrees, two frontiers and a
- * control block, about 12 MiB) is a fixed array that every GPU loading the
+ * without allocating anything: its scratch (peel degrees, removal order, near list
+ * and a control block, about 12 MiB) is a fixed array that every GPU loading the
  * library holds until the process exits.
  * n: vertices, at most KCL_NOALLOC_MAX_VERTICES (else KCL_ESIZE, nothing run).
  * row_ptr, col: the symmetric CSR graph in device memory (as for

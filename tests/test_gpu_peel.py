@@ -1,7 +1,7 @@
-"""The degeneracy peel's rounds against the oracle where its rules change:
-grid and cluster (handover above 2^17 vertices), thresholds past the near
-list's window and gaps wider than it, rows longer than 4,096 in wide rounds,
-and more of those than a round's list holds.  Both entry points."""
+"""The degeneracy peel's rounds against the oracle where its rules change: one
+CTA, one cluster, grid and cluster, thresholds past the near list's window and
+gaps wider than it, rows longer than 4,096 in wide rounds, and more of those
+than a round's list holds.  Both entry points."""
 import numpy as np
 import pytest
 
@@ -37,7 +37,9 @@ def _cliques(*sizes):
 
 
 GRAPHS = {
-    "grid_and_cluster": lambda: kclgen.rmat20(seed=5, scale=18),
+    "cluster": lambda: kclgen.rmat20(seed=5, scale=18),
+    "grid_and_cluster": lambda: kclgen.rmat20(seed=6, scale=19),
+    "one_cta": lambda: kclgen.chung_lu(3000, 12000, 2.3, groups=5, group_size=(10, 40), seed=4),
     "gaps": lambda: _cliques(20, 53, 55, 150, 400),
     "long_rows": lambda: _layers(5, 1, 2),
     "many_long_rows": lambda: _layers(300, 41, 42),
