@@ -1,16 +1,16 @@
 // C ABI of the library (include/kcl.h): graph loading and validation, and the
 // host-side orchestration of one k-clique call:
-//   stage 0  Pre-Core (Algorithm 3): frontier rounds until no vertex falls
-//            below degree k-1;
+//   stage 0  Pre-Core (Algorithm 3): vertices below degree k-1 removed until
+//            none is left, in one cooperative launch;
 //   stage 1  Pre-List (Algorithm 4): clique components counted by C(n_c, k)
 //            (and enumerated in listing mode), then removed;
 //   stage 2  orientation: degree key (Section VI-B) or degeneracy peel rounds
 //            (Algorithm 6), out-neighbour CSR, roots sorted by out-degree;
-//   stage 3  listing kernels: SDegreeList (Algorithm 5) or subgraph build +
-//            colouring + BitColList (Algorithm 6), one launch per out-degree
-//            class.
-// Every kernel runs on the graph's stream; the host reads back small status
-// words between stages (frontier sizes, Delta, class boundaries).
+//   stage 3  listing kernels, one launch per out-degree class: id-ordered
+//            subproblems for k <= 6, else SDegreeList (Algorithm 5) or subgraph
+//            build + colouring + BitColList (Algorithm 6).
+// Every kernel runs on the graph's stream; the host reads back one small status
+// record before stage 3 (Delta, class boundaries, the peel's error word).
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>

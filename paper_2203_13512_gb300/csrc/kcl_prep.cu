@@ -2,8 +2,8 @@
 // Pre-Core (Algorithm 3), Pre-List (Algorithm 4), the two orientations
 // (degree ordering of Section VI-B, degeneracy ordering of Algorithm 6) and
 // the out-neighbour CSR of the DAG, plus the root list the listing kernels
-// consume.  Every pass here streams the CSR once: these kernels are bound by
-// HBM bandwidth, so they use warp-per-vertex row scans with coalesced loads.
+// consume.  Most passes stream the CSR once with warp-per-vertex row scans and
+// coalesced loads; the peel is a chain of rounds, bound by the latency of each.
 #include <algorithm>
 #include <mutex>
 
