@@ -68,12 +68,18 @@ struct kcl_server {
 
 namespace {
 
-// Device scratch a query may need: the per-call workspace (about 70 bytes
-// per vertex and 2 per CSR entry) plus the listing kernels' arena bound.
+// Device scratch a query may need: the per-call workspace (74 bytes per
+// vertex, 2 per CSR entry and its fixed parts) plus the listing kernels'
+// arena bound.  The id-ordered kernels take more than the others at d+ near
+// 256 and 512; their need is not monotone in d+, but this bound covers every
+// d+ up to the maximum degree (compared for d+ up to 5,000).
 uint64_t scratch_estimate(const kcl_server *s, const kcl_graph *g, uint32_t k) {
-    uint64_t ws = 72ull * ((uint64_t)g->n + 1) + 2ull * g->nnz + (1u << 20);
+    uint64_t ws = 76ull * ((uint64_t)g->n + 1) + 2ull * g->nnz + (1u << 20);
     uint64_t arena = 4ull * std::max(kcl::bitcol_arena_words(k, s->num_sms, g->max_deg),
                                      kcl::sdegree_arena_words(k, s->num_sms, g->max_deg));
+    if (k <= 6)
+        for (bool listing : {false, true})
+            arena = std::max<uint64_t>(arena, 4ull * kcl::sub_arena_words(k, s->num_sms, g->max_deg, listing));
     return ws + arena;
 }
 
