@@ -1,7 +1,7 @@
 // C ABI of the library (include/kcl.h): graph loading and validation, and the
 // host-side orchestration of one k-clique call:
 //   stage 0  Pre-Core (Algorithm 3): vertices below degree k-1 removed until
-//            none is left, in one cooperative launch;
+//            none is left, a few launches of frontier rounds;
 //   stage 1  Pre-List (Algorithm 4): clique components counted by C(n_c, k)
 //            (and enumerated in listing mode), then removed;
 //   stage 2  orientation: degree key (Section VI-B) or degeneracy peel rounds
@@ -312,58 +312,37 @@ bool run_peel(kcl_graph *g, StageTimer &T) {
     return true;
 }
 
-// Stages 0-2.  listing: enumerate Pre-List cliques into the ring.
-kcl_status run_front(kcl_graph *g, uint32_t k, kcl_ordering ord, const kcl_ring *ring, bool listing,
-                     StageTimer &T, FrontEnd &fe) {
+// Stages 1 and 2 on the graph that Pre-Core left: one host read at the end, in the
+// pinned mirror (listing: one more, of the number of components to enumerate).
+// Leaves early, with a mirror that says so (pre_nin), when Pre-Core has rounds left.
+kcl_status run_orientation(kcl_graph *g, uint32_t k, kcl_ordering ord, const kcl_ring *ring, bool listing,
+                           StageTimer &T, FrontEnd &fe) {
     Workspace &w = g->ws;
     cudaStream_t s = g->stream;
-    KCL_TRY(ensure_workspace(g));
-    KCL_CK(cudaMemsetAsync(w.res, 0, sizeof(DevResult), s));
-    const uint32_t n = g->n;
-
-    // ---- stage 0: Pre-Core
-    T.begin(0);
-    // without Pre-Core the threshold is 0: every vertex stays
-    const uint32_t kcore = (g->options & KCL_OPT_NO_PRECORE) ? 1u : k;
-    uint32_t *fa = w.frontier_a, *fb = w.frontier_b;
-    if (const int l = launch_precore(g, kcore, w, s); l > 0) {
-        T.add(0, l);
-    } else {  // no co-resident launch here: one launch per round
-        (void)cudaGetLastError();
-        T.add(0, launch_precore_init(g, kcore, w, s));
-        for (;;) {
-            uint32_t nin = 0;
-            KCL_TRY(read_u32(g, &w.res->frontier, &nin));
-            if (nin == 0) break;
-            KCL_TRY(set_u32(g, &w.res->frontier, 0));
-            T.add(0, launch_precore_round(g, k, fa, nin, fb, w, s));
-            std::swap(fa, fb);
-        }
-    }
-    KCL_CK(cudaMemcpyAsync(w.alive_core, w.alive, n, cudaMemcpyDeviceToDevice, s));
-    T.end(0);
 
     // ---- stage 1: Pre-List
     T.begin(1);
     if (!(g->options & KCL_OPT_NO_PRELIST)) T.add(1, launch_prelist(g, k, w, listing ? 1 : 0, s));
     if (listing && !(g->options & KCL_OPT_NO_PRELIST)) {
-        uint32_t ncomp = 0;
-        KCL_TRY(read_u32(g, &w.res->n_clique_comps, &ncomp));
-        T.add(1, launch_prelist_emit(g, k, w, ncomp, ring, s));
+        KCL_TRY(read_result(g));
+        if (w.h_res->pre_nin) return KCL_OK;
+        T.add(1, launch_prelist_emit(g, k, w, w.h_res->n_clique_comps, ring, s));
     }
     T.end(1);
 
     // ---- stage 2: orientation
     T.begin(2);
+    const PeelCtl *peel = nullptr;
     if (ord == KCL_ORDER_DEGREE) {
         T.add(2, launch_degree_key(g, w, s));
-    } else if (!run_peel(g, T)) {
+    } else if (run_peel(g, T)) {
+        peel = w.peel;
+    } else {
         T.add(2, launch_peel_init(g, w, s));
         uint32_t remaining = 0;
         KCL_TRY(read_u32(g, &w.res->remaining, &remaining));
         uint32_t t = 0, round = 0, nin = 0;
-        fa = w.frontier_a;
-        fb = w.frontier_b;
+        uint32_t *fa = w.frontier_a, *fb = w.frontier_b;
         while (remaining > 0) {
             if (nin == 0) {
                 KCL_TRY(set_u32(g, &w.res->min_deg, 0xFFFFFFFFu));
@@ -389,9 +368,37 @@ kcl_status run_front(kcl_graph *g, uint32_t k, kcl_ordering ord, const kcl_ring 
     T.add(2, launch_orient(g, k, w, s));
     uint32_t *limits = fe.limits;
     fe.n_classes = ord == KCL_ORDER_DEGREE ? sdegree_classes(limits, 16) : bitcol_classes(limits, 16);
-    T.add(2, launch_roots(g, k, w, limits, fe.n_classes, s));
+    T.add(2, launch_roots(g, k, w, limits, fe.n_classes, peel, s));
     T.end(2);
-    KCL_TRY(read_result(g));
+    return read_result(g);
+}
+
+// Stages 0-2.  listing: enumerate Pre-List cliques into the ring.
+kcl_status run_front(kcl_graph *g, uint32_t k, kcl_ordering ord, const kcl_ring *ring, bool listing,
+                     StageTimer &T, FrontEnd &fe) {
+    Workspace &w = g->ws;
+    cudaStream_t s = g->stream;
+    KCL_TRY(ensure_workspace(g));
+    KCL_CK(cudaMemsetAsync(w.res, 0, sizeof(DevResult), s));
+
+    // ---- stage 0: Pre-Core
+    T.begin(0);
+    // without Pre-Core the threshold is 0: every vertex stays
+    const uint32_t kcore = (g->options & KCL_OPT_NO_PRECORE) ? 1u : k;
+    T.add(0, launch_precore(g, kcore, w, s));
+    T.end(0);
+    for (;;) {
+        KCL_CK(cudaMemcpyAsync(w.alive_core, w.alive, g->n, cudaMemcpyDeviceToDevice, s));
+        KCL_TRY(run_orientation(g, k, ord, ring, listing, T, fe));
+        if (w.h_res->pre_nin == 0) break;
+        // more wide rounds than Pre-Core's launches: nothing has been counted,
+        // listed or removed since (k_pl_check), so the rest follows once they are done
+        for (uint32_t nin = 1; nin;) {
+            T.add(0, launch_precore_rounds(g, kcore, w, 8, s));
+            KCL_TRY(read_u32(g, &w.res->pre_nin, &nin));
+        }
+        KCL_CK(cudaMemsetAsync(w.res, 0, sizeof(DevResult), s));
+    }
     if (w.h_res->peel_error) return KCL_ETIMEOUT;
     fe.max_outdeg = w.h_res->max_outdeg;
     fe.n_roots = w.h_res->n_roots;
@@ -400,7 +407,6 @@ kcl_status run_front(kcl_graph *g, uint32_t k, kcl_ordering ord, const kcl_ring 
     if (w.h_res->status) return status_from_device(w.h_res->status);
     // roots above the largest class cannot be processed
     if (fe.class_begin[fe.n_classes - 1] > 0) return KCL_ELIMIT;
-    (void)listing;
     return KCL_OK;
 }
 

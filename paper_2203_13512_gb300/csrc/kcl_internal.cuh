@@ -38,7 +38,10 @@ struct DevResult {
     unsigned int min_deg;            // minimum current degree (degeneracy peel)
     unsigned int remaining;          // vertices not yet peeled
     unsigned int n_clique_comps;     // components removed by Pre-List
-    unsigned int peel_error;         // error word of Pre-Core's or the peel's barriers
+    unsigned int peel_error;         // error word of the peel's barriers
+    unsigned int pre_lo, pre_nin;    // Pre-Core: the current frontier's place in the list and its size
+    unsigned int pre_next;           // Pre-Core: the next frontier's size so far
+    unsigned int pre_finished;       // Pre-Core: blocks of the launch that are done
     unsigned long long deadline_ns;  // %globaltimer value after which listing stops (0: none)
     unsigned int class_begin[KCL_MAX_CLASSES + 1];  // root positions where the out-degree classes start
 };
@@ -110,7 +113,7 @@ struct Workspace {
     uint32_t *hist = nullptr;        // histogram / scan scratch
     uint32_t *scan_tmp = nullptr;    // block sums for scans
     unsigned int *queue = nullptr;   // per-class work counters
-    uint32_t *members = nullptr;     // n: clique-component members (listing)
+    uint32_t *members = nullptr;     // n: vertices that left in Pre-Core, then clique-component members (listing)
     uint32_t *comp_slot = nullptr;   // n: clique-component slot (listing)
     uint32_t *arena = nullptr;       // global scratch for large subproblems
     uint32_t *small_arena = nullptr; // the arena of calls that need almost none
@@ -527,12 +530,10 @@ inline bool allow_max_smem(K kern) {
 // kcl_prep.cu
 int launch_validate(const kcl_graph *g, DevResult *res, cudaStream_t s);
 int launch_degrees(const kcl_graph *g, uint32_t *deg, cudaStream_t s);
-// All of Pre-Core in one launch of co-resident blocks (clears w.peel first); -1
-// if it cannot launch.
+// Pre-Core (res zeroed first): the initial frontier and a few rounds; res->pre_nin
+// is the frontier that is left, 0 almost always.  launch_precore_rounds: more rounds.
 int launch_precore(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s);
-int launch_precore_init(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s);
-int launch_precore_round(const kcl_graph *g, uint32_t k, const uint32_t *fin, uint32_t nin,
-                         uint32_t *fout, Workspace &w, cudaStream_t s);
+int launch_precore_rounds(const kcl_graph *g, uint32_t k, Workspace &w, int rounds, cudaStream_t s);
 int launch_prelist(const kcl_graph *g, uint32_t k, Workspace &w, int listing, cudaStream_t s);
 int launch_prelist_emit(const kcl_graph *g, uint32_t k, Workspace &w, uint32_t n_comps,
                         const kcl_ring *ring, cudaStream_t s);
@@ -548,8 +549,9 @@ int launch_peel_min(const kcl_graph *g, Workspace &w, cudaStream_t s);
 int launch_peel(const kcl_graph *g, Workspace &w, cudaStream_t s);
 int launch_orient(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s);
 // Roots by descending out-degree; res->class_begin, n_roots and peel_error.
+// peel: the control block of a co-resident peel, or null.
 int launch_roots(const kcl_graph *g, uint32_t k, Workspace &w, const uint32_t *class_limits, int n_classes,
-                 cudaStream_t s);
+                 const PeelCtl *peel, cudaStream_t s);
 int launch_exclusive_scan(const uint32_t *in, uint32_t *out, uint32_t n, uint32_t *block_tmp,
                           cudaStream_t s);
 // res->deadline_ns = now + limit_ms (or 0 when limit_ms is 0).

@@ -121,89 +121,6 @@ __global__ void k_validate(uint32_t n, uint64_t nnz, const uint64_t *__restrict_
 }
 
 // ------------------------------------------------------------- Pre-Core
-// Algorithm 3, frontier form: the initial queue is every vertex of degree
-// < k-1; each round, every queued vertex lowers the degree of its alive
-// neighbours and a neighbour whose degree falls from k-1 to k-2 joins the
-// next queue (exactly one thread sees that transition).
-// thr = k-1, or per vertex kmap[v] - 1 when a k map is given (batches of
-// graphs with different k).
-__global__ void k_precore_init(uint32_t n, const uint64_t *__restrict__ rp, uint32_t thr,
-                               const uint8_t *__restrict__ kmap, uint8_t *alive, uint32_t *cdeg,
-                               uint32_t *fout, unsigned *fcount) {
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        uint32_t d = (uint32_t)(rp[v + 1] - rp[v]);
-        cdeg[v] = d;
-        bool keep = d >= (kmap ? kmap[v] - 1u : thr);
-        alive[v] = keep ? 1 : 0;
-        if (!keep) fout[atomicAdd(fcount, 1u)] = v;
-    }
-}
-
-__global__ void k_precore_round(const uint64_t *__restrict__ rp, const uint32_t *__restrict__ col,
-                                uint32_t thr, const uint8_t *__restrict__ kmap,
-                                const uint32_t *__restrict__ fin, uint32_t nin,
-                                uint8_t *alive, uint32_t *cdeg, uint32_t *fout, unsigned *fcount) {
-    const unsigned lane = lane_id();
-    for (uint32_t i = warp_global(); i < nin; i += warps_total()) {
-        uint32_t v = fin[i];
-        for (uint64_t e = rp[v] + lane; e < rp[v + 1]; e += 32) {
-            uint32_t w = col[e];
-            if (!alive[w]) continue;
-            uint32_t old = atomicSub(&cdeg[w], 1u);
-            if (old == (kmap ? kmap[w] - 1u : thr)) {  // fell from k-1 to k-2
-                alive[w] = 0;
-                fout[atomicAdd(fcount, 1u)] = w;
-            }
-        }
-    }
-}
-
-// The same in one launch of co-resident blocks: a grid barrier (about 2 us)
-// separates the rounds instead of a launch and a host read of the next
-// frontier's size (about 15 us): 0.12 -> 0.03 ms on a 2,000-vertex graph of five
-// rounds.  Vertices leave through one list (fout), a round's frontier being a
-// range of it; its size counters rotate over three rounds as in the peel below.
-constexpr unsigned long long kSpinLimit = 1ull << 25;
-
-__device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ unsigned atom_add_acq_rel(unsigned *p, unsigned x) {
-    unsigned old;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(x) : "memory");
-    return old;
-}
-
-// Generation barrier: thread 0 of each block arrives with an acquire-release
-// add (publishing the block's writes, which __syncthreads has ordered before
-// it); the last arrival clears the count and bumps the generation with a
-// release, and the others poll the generation with acquire loads.
-__device__ bool grid_barrier(PeelCtl *c, unsigned nblocks) {
-    __shared__ int ok_s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const unsigned g = ld_acquire(&c->bar_gen);
-        const unsigned arrived = atom_add_acq_rel(&c->bar_count, 1u);
-        int ok = 1;
-        if (arrived == nblocks - 1) {
-            atomicExch(&c->bar_count, 0u);
-            atom_add_acq_rel(&c->bar_gen, 1u);
-        } else {
-            unsigned long long spins = 0;
-            while (ld_acquire(&c->bar_gen) == g) {
-                if (ld_acquire(&c->error)) { ok = 0; break; }
-                if (++spins > kSpinLimit) { atomicExch(&c->error, 1u); ok = 0; break; }
-            }
-        }
-        ok_s = ok && ld_acquire(&c->error) == 0;
-    }
-    __syncthreads();
-    return ok_s != 0;
-}
-
 // One warp's lanes append to a list: the position of this lane's entry.
 __device__ __forceinline__ uint32_t warp_append(unsigned m, unsigned *count) {
     const unsigned lane = lane_id();
@@ -212,13 +129,29 @@ __device__ __forceinline__ uint32_t warp_append(unsigned m, unsigned *count) {
     return __shfl_sync(0xffffffffu, base, 0) + __popc(m & ((1u << lane) - 1u));
 }
 
-__global__ void __launch_bounds__(1024) k_precore(uint32_t n, const uint64_t *__restrict__ rp,
-                                                 const uint32_t *__restrict__ col, uint32_t thr,
-                                                 const uint8_t *__restrict__ kmap, uint8_t *alive,
-                                                 uint32_t *cdeg, uint32_t *fout, PeelCtl *c, DevResult *res) {
-    const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+// Algorithm 3, frontier form: the first frontier is every vertex of degree
+// < k-1; each round, every vertex of the frontier lowers the degree of its
+// neighbours, and a neighbour whose degree falls from k-1 to k-2 joins the next
+// one (exactly one thread sees that transition; a vertex that left has fallen
+// below its threshold, so nobody sees it again).  Vertices leave through one list,
+// a round's frontier being a range of it.
+// thr = k-1, or per vertex kmap[v] - 1 when a k map is given (batches of
+// graphs with different k).
+// Launches are ordinary ones and no block waits for another.  In one cooperative
+// launch of co-resident blocks Pre-Core had to wait for room on every SM at once:
+// beside a k = 9 call on another stream a k = 5 degree count of the 131k-vertex R-MAT
+// graph took as long as that call (2.2 s), and takes 4.2 ms this way.  Short rounds
+// would cost a launch each; instead a launch's last block to finish runs the rounds
+// that follow while they have at most kPreTail vertices, and leaves wider ones to
+// the next launch (k = 5 count of a 2,000-vertex graph: 214 -> 206 us).
+constexpr uint32_t kPreTail = 2048;
+constexpr int kPreThreads = 512;
+
+__global__ void k_precore_init(uint32_t n, const uint64_t *__restrict__ rp, uint32_t thr,
+                               const uint8_t *__restrict__ kmap, uint8_t *alive, uint32_t *cdeg,
+                               uint32_t *list, DevResult *res) {
     const unsigned lane = lane_id();
-    volatile PeelCtl *vc = c;
+    const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
     for (uint32_t v0 = tid - lane; v0 < n; v0 += nth) {  // warp-uniform trip count
         const uint32_t v = v0 + lane;
         bool out = false;
@@ -230,47 +163,100 @@ __global__ void __launch_bounds__(1024) k_precore(uint32_t n, const uint64_t *__
         }
         const unsigned m = __ballot_sync(0xffffffffu, out);
         if (m) {
-            const uint32_t at = warp_append(m, &c->cnt.fcnt[0]);
-            if (out) fout[at] = v;
+            const uint32_t at = warp_append(m, &res->pre_nin);
+            if (out) list[at] = v;
         }
     }
-    auto barrier = [&]() {  // false: a wait gave up (the peel clears c, so the call's status takes it)
-        const bool ok = grid_barrier(c, gridDim.x);
-        if (!ok && threadIdx.x == 0) atomicOr(&res->status, DEV_ERR_TIMEOUT);
-        return ok;
-    };
-    if (!barrier()) return;
-    uint32_t round = 0, done = 0;
-    for (;;) {
-        const uint32_t nin = vc->cnt.fcnt[round % 3u];
-        if (nin == 0) return;
-        if (tid == 0) c->cnt.fcnt[(round + 2u) % 3u] = 0;
-        unsigned *next = &c->cnt.fcnt[(round + 1u) % 3u];
-        for (uint32_t i = tid >> 5; i < nin; i += nth >> 5) {
-            const uint32_t v = __ldcg(&fout[done + i]);
-            const uint64_t e = rp[v + 1];
-            for (uint64_t x = rp[v]; x < e; x += 32) {
-                uint32_t w = 0;
-                bool out = false;
-                if (x + lane < e) {
-                    w = col[x + lane];
-                    // a vertex that left has fallen below its threshold, so nobody sees the step again
-                    const uint32_t t = kmap ? kmap[w] - 1u : thr;
-                    out = t > 0 && atomicSub(&cdeg[w], 1u) == t;  // fell from k-1 to k-2
-                }
-                const unsigned m = __ballot_sync(0xffffffffu, out);
-                if (m) {
-                    const uint32_t at = warp_append(m, next);
-                    if (out) {
-                        alive[w] = 0;
-                        fout[done + nin + at] = w;
-                    }
-                }
-            }
+}
+
+struct PreArgs {
+    const uint64_t *rp;
+    const uint32_t *col;
+    uint32_t thr;
+    const uint8_t *kmap;
+    uint8_t *alive;
+    uint32_t *cdeg;
+    uint32_t *list;  // every vertex that left, in the order of the rounds
+    DevResult *res;
+};
+
+// One entry a lane (`in`: it has one): the neighbour loses a degree and may leave.
+__device__ __forceinline__ void precore_entry(const PreArgs &a, uint64_t x, bool in, uint32_t at, unsigned *next) {
+    uint32_t w = 0;
+    bool out = false;
+    if (in) {
+        w = a.col[x];
+        const uint32_t t = a.kmap ? a.kmap[w] - 1u : a.thr;
+        out = t > 0 && atomicSub(&a.cdeg[w], 1u) == t;  // fell from k-1 to k-2
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, out);
+    if (m) {
+        const uint32_t i = warp_append(m, next);
+        if (out) {
+            a.alive[w] = 0;
+            a.list[at + i] = w;
         }
-        done += nin;
-        round++;
-        if (!barrier()) return;
+    }
+}
+
+// The round of list[lo, lo + nin) by W warps, this one being number gw; the next
+// round is appended behind it.  Most rows are shorter than k: 8 lanes a row, and
+// the warp together for rows beyond 64 entries.
+__device__ void precore_round(const PreArgs &a, uint32_t lo, uint32_t nin, unsigned *next, uint32_t gw, uint32_t W) {
+    const unsigned lane = lane_id();
+    const uint32_t at = lo + nin;
+    for (uint32_t i0 = gw * 4; i0 < nin; i0 += W * 4) {
+        const uint32_t i = i0 + (lane >> 3);
+        uint64_t b = 0, e = 0;
+        if (i < nin) {
+            const uint32_t v = __ldcg(&a.list[lo + i]);
+            b = a.rp[v];
+            e = a.rp[v + 1];
+        }
+        const bool big = e - b > 64;
+        const uint32_t most = __reduce_max_sync(0xffffffffu, big ? 0u : (uint32_t)(e - b));
+        for (uint32_t x = lane & 7u; x - (lane & 7u) < most; x += 8)
+            precore_entry(a, b + x, !big && b + x < e, at, next);
+        for (unsigned todo = __ballot_sync(0xffffffffu, big && (lane & 7u) == 0); todo; todo &= todo - 1) {
+            const int j = __ffs(todo) - 1;
+            const uint64_t rb = __shfl_sync(0xffffffffu, b, j), re = __shfl_sync(0xffffffffu, e, j);
+            for (uint64_t x = rb; x < re; x += 32) precore_entry(a, x + lane, x + lane < re, at, next);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kPreThreads) k_precore_round(const PreArgs a) {
+    __shared__ unsigned next_s, last_s;
+    // changed only by the last block, when every block has read them
+    uint32_t lo = *(volatile unsigned *)&a.res->pre_lo, nin = *(volatile unsigned *)&a.res->pre_nin;
+    if (nin == 0) return;
+    const uint32_t W = blockDim.x >> 5, warp = threadIdx.x >> 5;
+    precore_round(a, lo, nin, &a.res->pre_next, blockIdx.x * W + warp, gridDim.x * W);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last_s = atomicAdd(&a.res->pre_finished, 1u) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last_s) return;
+    lo += nin;
+    nin = *(volatile unsigned *)&a.res->pre_next;
+    while (nin && nin <= kPreTail) {
+        __syncthreads();
+        if (threadIdx.x == 0) next_s = 0;
+        __syncthreads();
+        precore_round(a, lo, nin, &next_s, warp, W);
+        __syncthreads();
+        lo += nin;
+        nin = next_s;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        a.res->pre_lo = lo;
+        a.res->pre_nin = nin;
+        a.res->pre_next = 0;
+        a.res->pre_finished = 0;
     }
 }
 
@@ -394,6 +380,7 @@ __global__ void k_pl_check(uint32_t n, uint32_t k, const uint8_t *__restrict__ k
                            uint32_t *comp_slot, unsigned long long *vcount, DevResult *res) {
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
         if (!alive[v] || parent[v] != v) continue;
+        if (res->pre_nin) continue;  // Pre-Core has rounds left: the call comes back here after them
         const unsigned long long nc = comp_n[v];
         if (nc != (unsigned long long)cdeg[v] + 1) continue;  // not all of N[v] passed
         bool ovf = false;
@@ -565,6 +552,47 @@ __global__ void k_peel_update(const uint64_t *__restrict__ rp, const uint32_t *_
                 fout[atomicAdd(fcount, 1u)] = w;
         }
     }
+}
+
+constexpr unsigned long long kSpinLimit = 1ull << 25;
+
+__device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ unsigned atom_add_acq_rel(unsigned *p, unsigned x) {
+    unsigned old;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(x) : "memory");
+    return old;
+}
+
+// Generation barrier: thread 0 of each block arrives with an acquire-release
+// add (publishing the block's writes, which __syncthreads has ordered before
+// it); the last arrival clears the count and bumps the generation with a
+// release, and the others poll the generation with acquire loads.
+__device__ bool grid_barrier(PeelCtl *c, unsigned nblocks) {
+    __shared__ int ok_s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned g = ld_acquire(&c->bar_gen);
+        const unsigned arrived = atom_add_acq_rel(&c->bar_count, 1u);
+        int ok = 1;
+        if (arrived == nblocks - 1) {
+            atomicExch(&c->bar_count, 0u);
+            atom_add_acq_rel(&c->bar_gen, 1u);
+        } else {
+            unsigned long long spins = 0;
+            while (ld_acquire(&c->bar_gen) == g) {
+                if (ld_acquire(&c->error)) { ok = 0; break; }
+                if (++spins > kSpinLimit) { atomicExch(&c->error, 1u); ok = 0; break; }
+            }
+        }
+        ok_s = ok && ld_acquire(&c->error) == 0;
+    }
+    __syncthreads();
+    return ok_s != 0;
 }
 
 // The same peel in one launch of co-resident blocks: rounds are separated by
@@ -1040,7 +1068,7 @@ __global__ void k_root_scatter(uint32_t n, uint32_t k, const uint32_t *__restric
 
 // res->class_begin[c] = first root position whose d+ <= limits[c] (roots are
 // in descending d+), i.e. the number of roots with d+ > limits[c]; the last
-// entry is the number of roots.  Also the error word of the co-resident launches.
+// entry is the number of roots.  Also the peel's error word (peel null: no co-resident peel).
 __global__ void k_class_bounds(const uint32_t *__restrict__ offs, uint32_t top, const ClassLimits limits,
                                int n_classes, const PeelCtl *peel, DevResult *res) {
     const int c = threadIdx.x;
@@ -1051,7 +1079,7 @@ __global__ void k_class_bounds(const uint32_t *__restrict__ offs, uint32_t top, 
     }
     if (c == 0) {
         res->class_begin[n_classes] = res->n_roots;
-        res->peel_error = peel->error;
+        res->peel_error = peel ? peel->error : 0u;
     }
 }
 
@@ -1183,20 +1211,27 @@ int launch_validate(const kcl_graph *g, DevResult *res, cudaStream_t s) {
     return 1;
 }
 
-int launch_precore_init(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s) {
-    int grid = grid_for(g->n, kBlock, g->num_sms);
-    // a threshold of 0 (k = 1: Pre-Core switched off) keeps every vertex, whatever the k map says
-    k_precore_init<<<grid, kBlock, 0, s>>>(g->n, g->rp, k - 1, k > 1 ? w.kmap : nullptr, w.alive,
-                                           w.cdeg, w.frontier_a, &w.res->frontier);
-    return 1;
+// The arrays and the threshold of a call's Pre-Core.  A threshold of 0 (k = 1:
+// Pre-Core switched off) keeps every vertex, whatever the k map says.  The list is
+// in an array that the stages up to the first host read leave alone.
+static PreArgs precore_args(const kcl_graph *g, uint32_t k, Workspace &w) {
+    return PreArgs{g->rp, g->col, k - 1, k > 1 ? w.kmap : nullptr, w.alive, w.cdeg, w.members, w.res};
 }
 
-int launch_precore_round(const kcl_graph *g, uint32_t k, const uint32_t *fin, uint32_t nin,
-                         uint32_t *fout, Workspace &w, cudaStream_t s) {
-    int grid = grid_for((uint64_t)nin * 32, kBlock, g->num_sms, 32);
-    k_precore_round<<<grid, kBlock, 0, s>>>(g->rp, g->col, k - 1, k > 1 ? w.kmap : nullptr, fin, nin,
-                                            w.alive, w.cdeg, fout, &w.res->frontier);
-    return 1;
+int launch_precore_rounds(const kcl_graph *g, uint32_t k, Workspace &w, int rounds, cudaStream_t s) {
+    const PreArgs a = precore_args(g, k, w);
+    const int grid = grid_for((uint64_t)g->n * 8, kPreThreads, g->num_sms, 4);  // 8 lanes a row
+    for (int i = 0; i < rounds; i++) k_precore_round<<<grid, kPreThreads, 0, s>>>(a);
+    return rounds;
+}
+
+int launch_precore(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s) {
+    const PreArgs a = precore_args(g, k, w);
+    k_precore_init<<<grid_for(g->n, kBlock, g->num_sms), kBlock, 0, s>>>(g->n, a.rp, a.thr, a.kmap, a.alive, a.cdeg,
+                                                                        a.list, a.res);
+    // wide rounds by size: 400,000 vertices at k = 10 have three of more than
+    // kPreTail vertices, R-MAT graphs up to 2^20 vertices one
+    return 1 + launch_precore_rounds(g, k, w, g->n <= kPreTail ? 1 : g->n <= (1u << 16) ? 2 : 3, s);
 }
 
 int launch_prelist(const kcl_graph *g, uint32_t k, Workspace &w, int listing, cudaStream_t s) {
@@ -1381,33 +1416,6 @@ int launch_peel(const kcl_graph *g, Workspace &w, cudaStream_t s) {
     return peel_launches(a, peel_blocks(g->num_sms, g->n), g->nnz, true, s);
 }
 
-int launch_precore(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s) {
-    static std::atomic<int> cached{-1};  // several host threads (server slots) call this
-    int per_sm = cached.load(std::memory_order_relaxed);
-    if (per_sm < 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_precore, kPeelThreads, 0) != cudaSuccess) {
-            (void)cudaGetLastError();
-            per_sm = 0;
-        }
-        cached.store(per_sm, std::memory_order_relaxed);
-    }
-    if (per_sm <= 0 || cudaMemsetAsync(w.peel, 0, sizeof(PeelCtl), s) != cudaSuccess) return -1;
-    // two CTAs per SM, none beyond one vertex or 8 entries a thread
-    const uint64_t need = (std::max<uint64_t>(g->n, g->nnz / 8) + kPeelThreads - 1) / kPeelThreads;
-    const uint64_t most = (uint64_t)g->num_sms * (per_sm < 2 ? per_sm : 2);
-    const int blocks = (int)(need < 1 ? 1 : need < most ? need : most);
-    uint32_t n = g->n, thr = k - 1;
-    const uint64_t *rp = g->rp;
-    const uint32_t *col = g->col;
-    // a threshold of 0 (k = 1: Pre-Core switched off) keeps every vertex, whatever the k map says
-    const uint8_t *kmap = k > 1 ? w.kmap : nullptr;
-    void *args[] = {&n, (void *)&rp, (void *)&col, &thr, (void *)&kmap, &w.alive, &w.cdeg, &w.frontier_a, &w.peel,
-                    &w.res};
-    if (cudaLaunchCooperativeKernel((const void *)k_precore, blocks, kPeelThreads, args, 0, s) != cudaSuccess)
-        return -1;
-    return 1;
-}
-
 int launch_orient(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s) {
     (void)k;
     int wgrid = grid_for((uint64_t)g->n * 32, kBlock, g->num_sms, 32);
@@ -1419,7 +1427,7 @@ int launch_orient(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s) 
 }
 
 int launch_roots(const kcl_graph *g, uint32_t k, Workspace &w, const uint32_t *class_limits, int n_classes,
-                 cudaStream_t s) {
+                 const PeelCtl *peel, cudaStream_t s) {
     int grid = grid_for(g->n, kBlock, g->num_sms);
     // out-degrees are below n; those above the largest class need no order
     const uint32_t top = std::min<uint32_t>(g->n, KCL_MAX_OUTDEG + 2);
@@ -1431,7 +1439,7 @@ int launch_roots(const kcl_graph *g, uint32_t k, Workspace &w, const uint32_t *c
     k_root_hist<<<grid, kBlock, 0, s>>>(g->n, k, w.outdeg, top, hist, w.root_mask, w.kmap, w.res);
     int l = 1 + launch_exclusive_scan(hist, offs, H, w.scan_tmp, s);
     k_root_scatter<<<grid, kBlock, 0, s>>>(g->n, k, w.outdeg, top, offs, fill, w.root_mask, w.kmap, w.roots);
-    k_class_bounds<<<1, 32, 0, s>>>(offs, top, limits, n_classes, w.peel, w.res);
+    k_class_bounds<<<1, 32, 0, s>>>(offs, top, limits, n_classes, peel, w.res);
     return l + 2;
 }
 
