@@ -612,7 +612,7 @@ __device__ bool grid_barrier(PeelCtl *c, unsigned nblocks) {
 //     cluster of at most 16 CTAs the long tail, with its hardware barrier and the
 //     counters in the first CTA's shared memory.
 // On the 1M-vertex R-MAT graph (678 rounds) this took the peel from 17.5 to 6.3
-// ms, about 7 us a round in the cluster, 3.4 us on 65k vertices.
+// ms, about 7 us a round in the cluster, 3.1 us on 65k vertices.
 // Every thread follows the same control flow, derived from counters read after
 // a barrier; frontier and big-row counters rotate over three rounds (round r
 // reads slot r % 3, appends to (r + 1) % 3 and clears (r + 2) % 3, which
@@ -623,7 +623,15 @@ __device__ bool grid_barrier(PeelCtl *c, unsigned nblocks) {
 constexpr int kNear = 32;                 // thresholds a near list covers
 constexpr uint32_t kBigRow = 4096;        // longer rows are walked by all warps
 constexpr int kGone = -(1 << 30);         // degree of a vertex that is not alive
-constexpr int kPeelThreads = 1024;
+// 768 threads of 40 registers, two loads a lane: the co-resident CTAs and clusters
+// have to find room beside the kernels of other streams, and 1,024 threads of 52
+// (four loads a lane) fitted only into almost empty SMs: beside a k = 7 listing a
+// colour count of the 262k-vertex R-MAT graph waited 2.2 s for that call's end,
+// now 0.28 s.  Alone: 262k vertices 2.62 ms both, 60k 1.42 -> 1.35, 2,000 vertices
+// in one CTA 0.141 -> 0.125; 1,024 threads capped at 32 registers spilled (2.87).
+constexpr int kPeelThreads = 768;
+constexpr int kPeelLoads = 2;
+constexpr uint64_t kFetchEntries = 1ull << 25;  // 128 MB of ids
 
 struct PeelArgs {
     uint32_t n;
@@ -699,20 +707,20 @@ struct LocalRows {
     __device__ __forceinline__ uint32_t entry(Pos x) const { return col[x]; }
 };
 
-// Lowers the degrees of up to four neighbours a lane (n of them valid, stride
+// Lowers the degrees of up to kPeelLoads neighbours a lane (n of them valid, stride
 // `step` from x) and appends those that reach t or B.
 template <typename R>
 __device__ __forceinline__ void peel_relax(const PeelArgs &a, const R &rows, PeelCounters *c, unsigned *next,
                                            uint32_t next0, typename R::Pos x, typename R::Pos e,
                                            typename R::Pos step, int t, int B, uint32_t round) {
-    uint32_t w[4];
-    int old[4];
+    uint32_t w[kPeelLoads];
+    int old[kPeelLoads];
 #pragma unroll
-    for (int z = 0; z < 4; z++) w[z] = x + z * step < e ? rows.entry(x + z * step) : 0xFFFFFFFFu;
+    for (int z = 0; z < kPeelLoads; z++) w[z] = x + z * step < e ? rows.entry(x + z * step) : 0xFFFFFFFFu;
 #pragma unroll
-    for (int z = 0; z < 4; z++) old[z] = w[z] != 0xFFFFFFFFu ? atomicSub(&a.deg[w[z]], 1) : kGone;
+    for (int z = 0; z < kPeelLoads; z++) old[z] = w[z] != 0xFFFFFFFFu ? atomicSub(&a.deg[w[z]], 1) : kGone;
 #pragma unroll
-    for (int z = 0; z < 4; z++) {
+    for (int z = 0; z < kPeelLoads; z++) {
         const bool join = old[z] == t + 1;
         const unsigned m = __ballot_sync(0xffffffffu, join);
         if (m) {
@@ -836,7 +844,7 @@ __device__ __forceinline__ bool peel_rounds(const PeelArgs &a, const R &rows, Pe
                 }
             }
             const Pos step = (Pos)32 << ls;
-            for (Pos x = b + 32 * (unit & ((1u << ls) - 1u)); x < e; x += 4 * step)
+            for (Pos x = b + 32 * (unit & ((1u << ls) - 1u)); x < e; x += kPeelLoads * step)
                 peel_relax(a, rows, c, next, next0, x + lane, e, step, st.t, st.B, st.round);
         }
         if (!sync()) return false;
@@ -845,7 +853,7 @@ __device__ __forceinline__ bool peel_rounds(const PeelArgs &a, const R &rows, Pe
             for (uint32_t i = 0; i < nb; i++) {
                 const uint32_t v = __ldcg(&big[i]);
                 const Pos b = rows.begin(v), e = rows.end(v);
-                for (Pos x = b + (Pos)gw * 32; x < e; x += (Pos)4 * nth)
+                for (Pos x = b + (Pos)gw * 32; x < e; x += (Pos)kPeelLoads * nth)
                     peel_relax(a, rows, c, next, next0, x + lane, e, nth, st.t, st.B, st.round);
             }
             if (!sync()) return false;
@@ -858,7 +866,7 @@ __device__ __forceinline__ bool peel_rounds(const PeelArgs &a, const R &rows, Pe
 }
 
 // The wide rounds, all SMs.
-__global__ void __launch_bounds__(1024) k_peel_grid(const PeelArgs a) {
+__global__ void __launch_bounds__(kPeelThreads, 2) k_peel_grid(const PeelArgs a) {
     PeelCounters *c = &a.ctl->cnt;
     const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
     const GridSync sync{a.ctl, gridDim.x};
@@ -867,10 +875,23 @@ __global__ void __launch_bounds__(1024) k_peel_grid(const PeelArgs a) {
     PeelState st{0, 0, 0, -1, -1, *(volatile unsigned *)&a.ctl->total};
     if (!peel_rounds<false>(a, GlobalRows{a.rp, a.col}, c, st, a.handover, tid, nth, sync)) return;
     if (tid == 0) a.ctl->st = st;
+    // The cluster reads the remaining rows on 16 SMs, most of them for the first
+    // time: all SMs fetch them into L2 before they leave (262k vertices 2.90 -> 2.74
+    // ms with nothing in L2 before, 65k 1.54 -> 1.45), if they fit there.
+    if (st.done == st.total || a.rp[a.n] > kFetchEntries) return;
+    const unsigned lane = lane_id();
+    for (uint32_t v0 = tid - lane; v0 < a.n; v0 += nth) {
+        const bool rest = v0 + lane < a.n && __ldcg(&a.deg[v0 + lane]) > st.t;
+        for (unsigned todo = __ballot_sync(0xffffffffu, rest); todo; todo &= todo - 1) {
+            const uint32_t v = v0 + __ffs(todo) - 1;
+            for (uint64_t x = a.rp[v] + 32 * lane; x < a.rp[v + 1]; x += 1024)
+                asm volatile("prefetch.global.L2 [%0];" :: "l"(a.col + x));
+        }
+    }
 }
 
 // The rest (or, for small graphs, all of it: resume = 0) in one cluster.
-__global__ void __launch_bounds__(1024) k_peel_cluster(const PeelArgs a, int resume) {
+__global__ void __launch_bounds__(kPeelThreads, 2) k_peel_cluster(const PeelArgs a, int resume) {
     __shared__ PeelCounters own;
     __shared__ unsigned total;
     uint32_t rank, csize;
@@ -913,11 +934,10 @@ __global__ void __launch_bounds__(1024) k_peel_cluster(const PeelArgs a, int res
 
 // Small graphs in one CTA, with the degrees, the removal order and the near
 // list in shared memory, and the rows too when they fit (LOCAL), so a round makes
-// no L2 round trip.  Orientation stage of a 2,000-vertex graph of 67 rounds: 0.22
-// ms in the cluster, 0.15 with the rows in global memory, 0.14 with all of it
-// here; of a 10,000-vertex graph of 100,000 entries 0.38 in the cluster, 0.44 here.
+// no L2 round trip.  Orientation stage of a 2,000-vertex graph of 67 rounds: 0.20
+// ms in the cluster, 0.14 with the rows in global memory, 0.13 with all of it here.
 template <bool LOCAL>
-__global__ void __launch_bounds__(1024) k_peel_block(PeelArgs a, uint32_t nnz) {
+__global__ void __launch_bounds__(kPeelThreads, 2) k_peel_block(PeelArgs a, uint32_t nnz) {
     extern __shared__ int peel_smem[];
     __shared__ PeelCounters own;
     __shared__ unsigned total;
@@ -1304,14 +1324,18 @@ int launch_peel_update(const kcl_graph *g, Workspace &w, const uint32_t *fin, ui
     return 1;
 }
 
-// Graphs up to this size are peeled in the cluster alone, and the grid leaves
-// the last kHandover vertices to it.  Orientation stage of the 1M-vertex and
-// the 262k-vertex R-MAT graph in ms: handover at 8k vertices 11.2 / 5.0, 32k
-// 10.4 / 3.6, 128k 9.2 / 3.2, 400k 9.3 / 3.2 (all cluster), the grid to the end
-// 10.4 / 5.4.
+// Up to kClusterVertices vertices and kClusterEntries entries one cluster does the
+// whole peel.  Of larger graphs the grid does the wide rounds, leaves the last
+// kHandover vertices to the cluster and fetches their rows for it; a graph of fewer
+// vertices but more entries it only sets up and fetches (65k vertices of 8M entries:
+// 2.75 -> 2.62 ms; of 2M entries 1.59 either way).  Orientation stage of the 262k- and
+// the 1M-vertex R-MAT graph in ms: handover at 8k vertices 4.14 / 8.74, 32k 3.02 / 8.28,
+// 128k 2.82 / 7.48, 400k (262k vertices: all cluster) 2.86 / 7.93, the grid to the
+// end 4.37 / 7.71.
 // Up to kBlockVertices (whose arrays fit in shared memory) and kBlockEntries one
-// CTA takes the whole peel.
-constexpr uint32_t kBlockVertices = 1u << 14;
+// CTA takes the whole peel: 5,000 vertices of 38k entries 0.22 ms against 0.29 in the
+// cluster, 8,000 of 61k 0.37 both, 16,000 of 62k 0.41 against 0.31.
+constexpr uint32_t kBlockVertices = 1u << 13;
 constexpr uint64_t kBlockEntries = 1ull << 16;
 constexpr size_t kBlockShared = 220 * 1024;
 constexpr uint32_t kClusterVertices = 1u << 17;

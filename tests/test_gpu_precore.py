@@ -51,27 +51,37 @@ def test_many_wide_rounds(width, layers):
     assert list(zip(*got)) == [oracle.plain(*other, 3), want]
 
 
-@pytest.mark.parametrize("order", ORDS)
-def test_calls_beside_a_long_one(order):
+# the long call: k = 9 counts, whose kernels leave whole SMs idle, and a k = 7
+# listing, whose kernels sit on every SM with half of its registers
+@pytest.mark.parametrize("order,scale,long_call,k", [
+    ("degree", 17, "kcl_count", 9), ("color", 17, "kcl_count", 9), ("color", 18, "kcl_list", 7)])
+def test_calls_beside_a_long_one(order, scale, long_call, k):
     """A call of a few ms on one stream while another stream's kernels run for 4 s
-    (k = 9 on R-MAT 18, cut by its time limit): it must not wait for their end."""
+    (R-MAT 18, cut by its time limit): it must not wait for their end."""
     import torch
     import paper_2203_13512_gb300 as kcl
     a, b = torch.cuda.Stream(), torch.cuda.Stream()
     with torch.cuda.stream(a):
         long_g = kcl.kcl_load_csr(*kclgen.rmat20(seed=1, scale=18))
     with torch.cuda.stream(b):
-        g = kcl.kcl_load_csr(*kclgen.rmat20(seed=2, scale=17))
+        g = kcl.kcl_load_csr(*kclgen.rmat20(seed=3, scale=scale))
     want = kcl.kcl_count(g, 5, order)
+
+    def run_long():
+        if long_call == "kcl_list":
+            kcl.kcl_list(long_g, k, "color", None)
+        else:
+            kcl.kcl_count(long_g, k, "degree")
+
     kcl.kcl_set_time_limit(long_g, 1)  # loads the kernels, which waits for running ones
     with pytest.raises(kcl.KclError):
-        kcl.kcl_count(long_g, 9, "degree")
+        run_long()
     kcl.kcl_set_time_limit(long_g, 4000)
     status = []
 
     def run():
         try:
-            kcl.kcl_count(long_g, 9, "degree")
+            run_long()
         except kcl.KclError as e:
             status.append(e.status)
 
@@ -84,4 +94,4 @@ def test_calls_beside_a_long_one(order):
     alive = t.is_alive()
     t.join()
     assert got == want and status == [kcl.KCL_ETIMEOUT]
-    assert alive and took < 1.0
+    assert alive and took < 2.0
