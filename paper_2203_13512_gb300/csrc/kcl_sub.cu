@@ -66,6 +66,7 @@ __host__ __device__ inline uint32_t set_room(uint32_t c, bool list) {
 // them.  Per warp: kBitmaps candidate bitmaps of W words, the extract masks
 // (8 W) and the room of the compacted set.
 constexpr uint32_t kBitmaps = 3;  // candidate sets of the path (k <= 6)
+constexpr uint32_t kMetaDeadline = 2;  // META: unit, children taken, deadline (2 words)
 constexpr uint32_t kQueue = 64;   // build: members found in a warp's out-lists, waiting for lookup
 struct Lay {
     uint32_t D, W, WP, NBR, META, A, X, RS, LEN, HK, HV, BM, Q, per_warp, room, total;
@@ -707,8 +708,16 @@ struct Sub {
     const uint32_t *A, *nbr;
     uint32_t WP, W, d, u, ru;
     uint32_t slice, slices;  // the share of a first-level child's own children this walk takes
-    unsigned long long deadline;
 };
+
+// The call's time limit, checked at every node that is walked (a first-level child
+// alone can take 50 ms: near-complete graph of 600 vertices, k = 6 listing).  The
+// deadline lies behind the members in shared memory, where it takes no registers,
+// and without a limit one uniform branch is all that is done.
+__device__ __forceinline__ bool late(const Sub &s, const SubArgs &a) {
+    const unsigned long long d = *reinterpret_cast<const unsigned long long *>(s.nbr + a.D + kMetaDeadline);
+    return d && warp_past_deadline(d, a.res);
+}
 
 // Candidate set of path vertex w below C (C null: all of N+_u): row(w) & C,
 // restricted to indices above w when rows are symmetric (UP).  Returns its size.
@@ -758,6 +767,7 @@ __device__ void walk(const Sub &s, uint32_t last, uint32_t c, uint32_t *path, co
                 if (J == 1 && at++ % s.slices != s.slice) continue;
                 const uint32_t n = next_set<LIST>(s, C, w, Cn);
                 if (n + J + 2 >= K) {  // K - J - 2 more vertices needed
+                    if (late(s, a)) return;
                     if (LIST) path[J] = s.nbr[w];
                     walk<K, J + 1, LIST>(s, w, n, path, sc, a, cnt, cks);
                 }
@@ -824,7 +834,9 @@ __device__ __forceinline__ void run(const SubArgs &a) {
     sc.gmem = a.gscratch + (size_t)(blockIdx.x * (blockDim.x >> 5) + wib) * a.gwords;
     const uint32_t units = (a.end - a.begin) * a.parts;
     const uint32_t nd = CTA && a.dfs_warps && a.dfs_warps < nwarps ? a.dfs_warps : nwarps;
-    const unsigned long long deadline = __ldcg(&a.res->deadline_ns);
+    unsigned long long &deadline = *reinterpret_cast<unsigned long long *>(meta + kMetaDeadline);
+    if (G::tid() == 0) deadline = __ldcg(&a.res->deadline_ns);
+    G::sync();
     unsigned long long cnt = 0, cks = 0;
     for (;;) {
         uint32_t unit;
@@ -850,7 +862,7 @@ __device__ __forceinline__ void run(const SubArgs &a) {
         if (!skip) {
             const Rows rows = LIST ? kBoth : k > 3 ? kLower : kNoRows;
             const uint32_t hits = build<CTA>(d, base, a, L, S, rows);
-            Sub s{S + L.A, S + L.NBR, L.WP, L.W, d, u, 0u, 0u, 1u, deadline};
+            Sub s{S + L.A, S + L.NBR, L.WP, L.W, d, u, 0u, 0u, 1u};
             if (LIST) {
                 uint32_t below = 0;  // members with an id below u
                 for (uint32_t i = lane; i < d; i += 32) below += s.nbr[i] < u ? 1u : 0u;
@@ -875,7 +887,7 @@ __device__ __forceinline__ void run(const SubArgs &a) {
                         if (lane == 0) i = atomicAdd(&meta[1], 1u);
                         i = __shfl_sync(kFull, i, 0);
                     }
-                    if (i >= nch * s.slices || warp_past_deadline(deadline, a.res)) break;
+                    if (i >= nch * s.slices || late(s, a)) break;
                     const uint32_t v = LIST ? part + i / s.slices * a.parts : d - 1 - part - i / s.slices * a.parts;
                     s.slice = i % s.slices;
                     if (k == 4) child<4, LIST>(s, v, sc, a, cnt, cks);

@@ -1,0 +1,40 @@
+"""The time limit inside the id-ordered kernels (k <= 6)."""
+import time
+
+import pytest
+
+import oracle
+from tests.graphs import gnp
+
+pytestmark = pytest.mark.gpu
+LIMIT_MS = 20
+
+
+# Between two looks at the timer lies one node: the triangles or the records of one
+# set of up to 600 members, well under 2 ms with every warp of an SM at work; the
+# front end, which has no limit, and the launches take about 1 ms.  10 ms over the
+# limit cover both; whole first-level children took 20 to 60 ms over it.
+@pytest.mark.parametrize("order", ["color", "degree"])
+@pytest.mark.parametrize("k,mode", [(5, "list"), (6, "count"), (6, "list")])
+def test_stops_within_a_node(k, mode, order):
+    import paper_2203_13512_gb300 as kcl
+    rp, col = gnp(600, 0.995, seed=1)
+    g = kcl.kcl_load_csr(rp, col)
+
+    def call():
+        if mode == "count":
+            kcl.kcl_count(g, k, order)
+        else:
+            kcl.kcl_list(g, k, order, None)
+
+    took = []
+    kcl.kcl_set_time_limit(g, LIMIT_MS)
+    for _ in range(4):  # the first one loads the kernels
+        start = time.perf_counter()
+        with pytest.raises(kcl.KclError) as e:
+            call()
+        took.append(1e3 * (time.perf_counter() - start))
+        assert e.value.status == kcl.KCL_ETIMEOUT
+    assert LIMIT_MS <= min(took) < LIMIT_MS + 10
+    kcl.kcl_set_time_limit(g, 600_000)
+    assert kcl.kcl_count(g, 4, order) == oracle.plain(rp, col, 4)[0]
