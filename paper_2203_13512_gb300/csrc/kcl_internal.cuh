@@ -482,29 +482,44 @@ __device__ __forceinline__ void hash_size(uint32_t d, uint32_t *T, uint32_t *shi
     *shift = 32 - lg;
 }
 
+// A value of at least 0 that is found once per device: device limits, occupancies and
+// function attributes belong to the device that is current when they are asked for
+// or set, and a process may use several.  Several host threads call this; find() may
+// run in more than one of them.
+class PerDevice {
+    std::atomic<int> cached_[64];  // value + 1, 0 = not yet found (static storage)
+
+public:
+    template <typename F>
+    int get(F find) {
+        int dev = -1;
+        if (cudaGetDevice(&dev) != cudaSuccess) (void)cudaGetLastError();
+        const bool keep = dev >= 0 && dev < 64;
+        if (keep) {
+            const int c = cached_[dev].load(std::memory_order_relaxed);
+            if (c) return c - 1;
+        }
+        const int v = find(dev);
+        if (keep) cached_[dev].store(v + 1, std::memory_order_relaxed);
+        return v;
+    }
+};
+
 // Largest dynamic shared memory a block may opt in to on the current device.
 // Kernels get their MaxDynamicSharedMemorySize attribute set to this value
 // (never to a call-specific size): the attribute is per-function state, and
 // calls running concurrently on several host threads must not shrink it
 // under each other.
 inline int max_dynamic_smem() {
-    static std::atomic<int> cached[64];  // 0 = not yet read (several host threads call this)
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) {
-        (void)cudaGetLastError();
-        dev = 0;
-    }
-    if (dev >= 0 && dev < 64) {
-        const int c = cached[dev].load(std::memory_order_relaxed);
-        if (c) return c;
-    }
-    int v = 48 * 1024;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
-        (void)cudaGetLastError();
-        v = 48 * 1024;
-    }
-    if (dev >= 0 && dev < 64) cached[dev].store(v, std::memory_order_relaxed);
-    return v;
+    static PerDevice limit;
+    return limit.get([](int dev) {
+        int v = 48 * 1024;
+        if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev < 0 ? 0 : dev) != cudaSuccess) {
+            (void)cudaGetLastError();
+            v = 48 * 1024;
+        }
+        return v;
+    });
 }
 
 // Let `kern` use as much dynamic shared memory as the device allows next to

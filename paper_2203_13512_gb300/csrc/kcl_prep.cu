@@ -1345,17 +1345,15 @@ constexpr uint32_t kHandover = 1u << 17;
 // Blocks of the grid's peel for n vertices: one per SM (fewer arrivals per
 // grid barrier), none beyond what n needs; -1 if it cannot be resident.
 int peel_blocks(int num_sms, uint32_t n) {
-    static std::atomic<int> cached{-1};  // several host threads (server slots) call this
-    int per_sm = cached.load(std::memory_order_relaxed);
-    if (per_sm < 0) {
+    static PerDevice resident;
+    const int per_sm = resident.get([](int) {
         int b = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_peel_grid, kPeelThreads, 0) != cudaSuccess) {
             (void)cudaGetLastError();
             b = 0;
         }
-        per_sm = b;
-        cached.store(b, std::memory_order_relaxed);
-    }
+        return b;
+    });
     if (per_sm <= 0) return -1;
     int blocks = num_sms;
     const uint64_t need = ((uint64_t)n + kPeelThreads - 1) / kPeelThreads;
@@ -1375,24 +1373,22 @@ static void cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, i
     cfg.numAttrs = 1;
 }
 
-// Largest cluster of the peel the device can place (16 CTAs need the
-// non-portable size), 0 if none.
+// Largest cluster of the peel the current device can place (16 CTAs need the
+// non-portable size, which is allowed on each device separately), 0 if none.
 static int peel_cluster_size() {
-    static std::atomic<int> cached{-1};
-    int best = cached.load(std::memory_order_relaxed);
-    if (best >= 0) return best;
-    best = 0;
-    (void)cudaFuncSetAttribute(k_peel_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    for (int size = 16; size >= 1 && !best; size >>= 1) {
-        cudaLaunchConfig_t cfg;
-        cudaLaunchAttribute attr;
-        cluster_config(cfg, attr, size, nullptr);
-        int fit = 0;
-        if (cudaOccupancyMaxActiveClusters(&fit, k_peel_cluster, &cfg) == cudaSuccess && fit > 0) best = size;
-        (void)cudaGetLastError();
-    }
-    cached.store(best, std::memory_order_relaxed);
-    return best;
+    static PerDevice largest;
+    return largest.get([](int) {
+        (void)cudaFuncSetAttribute(k_peel_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        for (int size = 16; size >= 1; size >>= 1) {
+            cudaLaunchConfig_t cfg;
+            cudaLaunchAttribute attr;
+            cluster_config(cfg, attr, size, nullptr);
+            int fit = 0;
+            if (cudaOccupancyMaxActiveClusters(&fit, k_peel_cluster, &cfg) == cudaSuccess && fit > 0) return size;
+            (void)cudaGetLastError();
+        }
+        return 0;
+    });
 }
 
 // The whole peel: wide rounds on the grid, the tail on one cluster.  nnz: the
