@@ -1050,8 +1050,9 @@ int launch_sub(const kcl_graph *g, uint32_t k, Workspace &w, int c, uint32_t beg
     uint32_t blocks = (uint32_t)g->num_sms * occ;
     // a class with few roots shares each root's children over several CTAs, which
     // all build it: up to 8 units per CTA of the launch (with up to 32, building
-    // took over: 131k k = 6 count 41.7 -> 60.6 ms; with up to 4, the tail: 43.1)
-    if (k >= 5 || (la.listing && k >= 4 && c >= kWarpClasses)) {
+    // took over: 131k k = 6 count 41.7 -> 60.6 ms; with up to 4, the tail: 43.1).
+    // dfs_warps = 1 asks for one warp per root (NodeParallel), so for no shares.
+    if (dfs_warps != 1 && (k >= 5 || (la.listing && k >= 4 && c >= kWarpClasses))) {
         while (a.parts < 8 && n * a.parts < 8 * blocks) a.parts *= 2;
     }
     if (blocks > n * a.parts) blocks = n * a.parts;

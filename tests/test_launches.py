@@ -17,10 +17,14 @@ def fake(tmp_path_factory):
     spec.loader.exec_module(b)
     b.build()
     objs = []
-    for src in ("kcl_prep.cu",):
+    for src in ("kcl_prep.cu", "kcl_sub.cu"):
         obj = os.path.join(b.BUILD, src + ".o")
         objs.append(obj if os.path.exists(obj) else b._compile(os.path.join(b.CSRC, src)))
-    lib = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    tmp = tmp_path_factory.mktemp("fake")
+    objs.append(str(tmp / "probe.o"))
+    subprocess.run([b.nvcc_path(), *b._flags(), "-c", os.path.join(ROOT, "tests", "launch_sub_probe.cu"), "-o",
+                    objs[-1]], check=True)
+    lib = str(tmp / "libfake.so")
     # symbols bound inside: the process may have the real runtime loaded as well
     subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic",
                     "-I" + os.path.join(os.path.dirname(os.path.dirname(b.nvcc_path())), "include"),
@@ -59,3 +63,16 @@ def test_peel_cluster_on_every_device(fake):
         assert _order(lib, 20_000) == 0
         assert [(d, k, b) for d, k, b, *_ in launches()] == [(dev, "k_peel_cluster", 16)]
     lib.fake_device(0)
+
+
+@pytest.mark.parametrize("k,c,listing", [(5, 4, 0), (6, 5, 0), (6, 1, 0), (4, 3, 1), (5, 2, 1), (6, 5, 1)])
+def test_one_warp_per_root_has_no_shares(fake, k, c, listing):
+    """A class of few roots: its roots are shared by several CTAs each, except when
+    one warp is to walk a root's whole subtree (NodeParallel)."""
+    lib, launches = fake
+    assert lib.probe_launch_sub(k, c, 10, 1024, listing, 0) == 1
+    (_, kernel, blocks, _, _), = launches()
+    assert kernel == "k_sub_cta" and 10 < blocks <= 80
+    assert lib.probe_launch_sub(k, c, 10, 1024, listing, 1) == 1
+    (_, kernel, blocks, _, _), = launches()
+    assert kernel == "k_sub_cta" and blocks == 10
