@@ -750,6 +750,7 @@ kcl_status kcl_count_roots(kcl_graph *g, uint32_t k, kcl_ordering ord, const uin
     if (cudaSetDevice(g->device) != cudaSuccess) return KCL_ECUDA;
     std::vector<uint8_t> mask((size_t)g->n + 1, 0);
     for (uint32_t i = 0; i < n_roots; i++) mask[roots[i]] = 1;
+    KCL_TRY(ensure_workspace(g));  // a new workspace (a view's first call) has no mask
     uint8_t *d_mask = nullptr;
     if (cudaMalloc((void **)&d_mask, mask.size()) != cudaSuccess) {
         (void)cudaGetLastError();
