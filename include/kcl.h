@@ -354,8 +354,9 @@ kcl_status kcl_set_tuning(kcl_graph *g, const kcl_tuning *t);
  * sdegree_bitmap first (candidates 0, 4, 64, 0xFFFFFFFF), then that mode's
  * galloping array (0, 40, 80, 160, 400); for both orderings it then tunes
  * that path's cta_warps array (0, 4, 8) and its split array (0, 2, 8, 32).
- * The tuning
- * is stored in g and copied to *out when out is not NULL.  Timing stays as
+ * Classes that the id-ordered kernels take (k <= 6) keep their galloping and split
+ * values, which those kernels do not use, and of the bitmap thresholds try only the
+ * other form (lists, or 0 where lists were set).  The tuning is stored in g and copied to *out when out is not NULL.  Timing stays as
  * the caller left it.  Errors: those of kcl_count / kcl_list. */
 kcl_status kcl_autotune(kcl_graph *g, uint32_t k, kcl_ordering ord, int listing, kcl_tuning *out);
 

@@ -16,6 +16,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <new>
@@ -982,29 +983,39 @@ kcl_status kcl_set_tuning(kcl_graph *g, const kcl_tuning *t) {
 namespace {
 
 // One tuning pass: for every candidate value of knob[] (all classes at once)
-// run the call and keep, per class, the fastest value.
+// run the call and keep, per class, the fastest value.  A class where reaches(c,
+// value) is false runs the same code as with its first value: nothing is tried there
+// (its timings would differ by chance only) and it keeps the value it had.
 kcl_status tune_knob(kcl_graph *g, uint32_t k, kcl_ordering ord, int listing, uint32_t *knob,
-                     const uint32_t *cand, int ncand) {
+                     const uint32_t *cand, int ncand, const std::function<bool(int, uint32_t)> &reaches) {
     float best_ms[KCL_MAX_CLASSES];
-    uint32_t best[KCL_MAX_CLASSES];
+    uint32_t best[KCL_MAX_CLASSES], own[KCL_MAX_CLASSES];
     for (int c = 0; c < KCL_MAX_CLASSES; c++) {
         best_ms[c] = -1.f;
-        best[c] = knob[c];
+        own[c] = best[c] = knob[c];
     }
     uint64_t cnt = 0, cks = 0, wr = 0;
     for (int i = 0; i < ncand; i++) {
-        for (int c = 0; c < KCL_MAX_CLASSES; c++) knob[c] = cand[i];
+        uint32_t tried[KCL_MAX_CLASSES];
+        bool any = i == 0;  // the first run also says which classes have roots
+        for (int c = 0; c < KCL_MAX_CLASSES; c++) {
+            tried[c] = reaches(c, cand[i]);
+            const bool roots = i == 0 || ((uint32_t)c < g->timing.n_classes && g->timing.class_roots[c]);
+            any = any || (tried[c] && roots);
+        }
+        if (!any) continue;
+        for (int c = 0; c < KCL_MAX_CLASSES; c++) knob[c] = tried[c] ? cand[i] : own[c];
         kcl_status st = listing ? kcl_list(g, k, ord, nullptr, &cnt, &cks, &wr) : kcl_count(g, k, ord, &cnt);
         if (st != KCL_OK) {
             for (int c = 0; c < KCL_MAX_CLASSES; c++) knob[c] = best[c];
             return st;
         }
         for (uint32_t c = 0; c < g->timing.n_classes && c < KCL_MAX_CLASSES; c++) {
-            if (!g->timing.class_roots[c]) continue;
+            if (!g->timing.class_roots[c] || (!tried[c] && best_ms[c] >= 0.f)) continue;
             const float ms = g->timing.class_ms[c];
             if (best_ms[c] < 0.f || ms < 0.98f * best_ms[c]) {
                 best_ms[c] = ms;
-                best[c] = cand[i];
+                best[c] = knob[c];
             }
         }
     }
@@ -1020,25 +1031,37 @@ kcl_status kcl_autotune(kcl_graph *g, uint32_t k, kcl_ordering ord, int listing,
     const int was_enabled = g->timing.enabled;
     KCL_TRY(kcl_enable_timing(g, 1));
     kcl_status st = KCL_OK;
+    // The id-ordered kernels have neither leaf forms nor the splitter, and of the
+    // bitmap thresholds only the list form leads elsewhere.
+    kcl_graph plain;
+    plain.options = g->options;
+    auto ranked = [&](int c, uint32_t) { return !sub_handles(g, k, c, ord); };
+    auto always = [](int, uint32_t) { return true; };
     if (ord == KCL_ORDER_DEGREE) {
         static const uint32_t bitmap_cand[] = {0, 4, 64, 0xFFFFFFFFu};
         static const uint32_t gallop_cand[] = {0, 40, 80, 160, 400};
-        st = tune_knob(g, k, ord, listing, g->tuning.sdegree_bitmap, bitmap_cand, 4);
+        uint32_t own[KCL_MAX_CLASSES];
+        memcpy(own, g->tuning.sdegree_bitmap, sizeof(own));
+        auto other_form = [&](int c, uint32_t v) {
+            const bool lists = v == 0xFFFFFFFFu, own_lists = own[c] == 0xFFFFFFFFu;
+            return !sub_handles(&plain, k, c, ord) || lists || (own_lists && v == 0);
+        };
+        st = tune_knob(g, k, ord, listing, g->tuning.sdegree_bitmap, bitmap_cand, 4, other_form);
         if (st == KCL_OK)
             st = tune_knob(g, k, ord, listing,
                            listing ? g->tuning.sdegree_gallop_list : g->tuning.sdegree_gallop,
-                           gallop_cand, 5);
+                           gallop_cand, 5, ranked);
     }
     static const uint32_t warps_cand[] = {0, 4, 8};
     if (st == KCL_OK)
         st = tune_knob(g, k, ord, listing,
                        ord == KCL_ORDER_DEGREE ? g->tuning.sdegree_cta_warps : g->tuning.bitcol_cta_warps,
-                       warps_cand, 3);
+                       warps_cand, 3, always);
     static const uint32_t split_cand[] = {0, 2, 8, 32};
     if (st == KCL_OK)
         st = tune_knob(g, k, ord, listing,
                        ord == KCL_ORDER_DEGREE ? g->tuning.sdegree_split : g->tuning.bitcol_split,
-                       split_cand, 4);
+                       split_cand, 4, ranked);
     if (!was_enabled) kcl_enable_timing(g, 0);
     if (st != KCL_OK) return st;
     if (out) *out = g->tuning;
