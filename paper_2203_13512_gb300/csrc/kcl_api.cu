@@ -963,7 +963,8 @@ kcl_status kcl_get_options(const kcl_graph *g, uint32_t *flags) {
 kcl_status kcl_scratch_bytes(const kcl_graph *g, uint64_t *workspace, uint64_t *arena) {
     if (!g || !workspace || !arena) return KCL_EINVAL;
     const Workspace &w = g->ws;
-    *workspace = w.slab_bytes;
+    // the small arena lies in the workspace's allocation; in use, it counts as arena
+    *workspace = w.slab_bytes - (w.arena && w.arena == w.small_arena ? kSmallArena * sizeof(uint32_t) : 0);
     *arena = (uint64_t)w.arena_words * 4;
     return KCL_OK;
 }
