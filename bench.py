@@ -897,16 +897,41 @@ def run_c3(args):
     return out
 
 
+def ablation_row(g, k, ordering, configs, repeats):
+    """Mean stage times of kcl_count on g for every (name, options, tuning) of configs."""
+    import torch
+
+    import paper_2203_13512_gb300 as kcl
+    row = {}
+    for name, flags, tune in configs:
+        kcl.kcl_set_options(g, flags)
+        kcl.kcl_set_tuning(g, tune or {})
+        c0 = kcl.kcl_count(g, k, ordering)  # warm-up
+        ms = []
+        for _ in range(max(1, repeats)):
+            torch.cuda.synchronize()
+            c = kcl.kcl_count(g, k, ordering)
+            assert c == c0
+            ms.append(kcl.kcl_last_timing(g)[0])
+        row[name] = {s_: round(sum(m[s_] for m in ms) / len(ms), 3) for s_ in ms[0]}
+        row[name]["count"] = c
+    return row
+
+
+PRUNE_K, PRUNE_SCALE = 7, 14  # BitCol's own kernels run k > 6
+
+
 def run_ablation(args):
     """The preprocessing / pruning study, the NodeParallel / EdgeParallel study
     and the memory study on the bench graph (R-MAT scale 20): for k = 4, 5
     and both orderings, device time of one call with everything on, without
-    Pre-Core, without Pre-List, (BitCol) without the colour prune, and with
-    one warp per root in the CTA classes (NodeParallel: no sharing of a
-    root's first-level children); and the device scratch a fresh handle holds
-    after one call of each (k, ordering)."""
-    import torch
-
+    Pre-Core, without Pre-List, and with one warp per root in the CTA classes
+    (NodeParallel: no sharing of a root's first-level children); and the device
+    scratch a fresh handle holds after one call of each (k, ordering).  The colour
+    prune, on and off, is compared at k = 7 on R-MAT scale 14, where both sides are
+    BitCol (for k <= 6 the id-ordered kernels have no colours, and switching the prune
+    off selects other kernels)."""
+    import kclgen
     import paper_2203_13512_gb300 as kcl
     rp, col = workload()
     g = kcl.kcl_load_csr(rp, col)
@@ -915,37 +940,25 @@ def run_ablation(args):
                 "bitcol_cta_warps": [1] * kcl.KCL_MAX_CLASSES}
     configs = [("all on", 0, None), ("no Pre-Core", kcl.KCL_OPT_NO_PRECORE, None),
                ("no Pre-List", kcl.KCL_OPT_NO_PRELIST, None),
-               ("no colour prune", kcl.KCL_OPT_NO_COLOR_PRUNE, None),
                ("one warp per root (NodeParallel)", 0, one_warp)]
     out = {"metric": "ablation: device ms per call (R-MAT scale 20)", "unit": "ms",
            "higher_is_better": False, "n_gpus": 1,
-           "config": {"workload": "rmat-scale20-ef16", "repeats": args.steps},
+           "config": {"workload": "rmat-scale20-ef16", "repeats": args.steps,
+                      "prune_workload": "rmat-scale%d-ef16" % PRUNE_SCALE},
            "data": "synthetic", "calls": {}, "scratch_bytes": {}}
     for k in (4, 5):
         for o in ("color", "degree"):
-            row = {}
-            for name, flags, tune in configs:
-                if o == "degree" and flags == kcl.KCL_OPT_NO_COLOR_PRUNE:
-                    continue
-                kcl.kcl_set_options(g, flags)
-                kcl.kcl_set_tuning(g, tune or {})
-                c0 = kcl.kcl_count(g, k, o)  # warm-up
-                ms = []
-                for _ in range(max(1, args.steps)):
-                    torch.cuda.synchronize()
-                    c = kcl.kcl_count(g, k, o)
-                    assert c == c0
-                    ms.append(kcl.kcl_last_timing(g)[0])
-                row[name] = {s_: round(sum(m[s_] for m in ms) / len(ms), 3) for s_ in ms[0]}
-                row[name]["count"] = c
-            out["calls"]["k=%d %s" % (k, o)] = row
+            out["calls"]["k=%d %s" % (k, o)] = ablation_row(g, k, o, configs, args.steps)
             v = kcl.kcl_graph_view(g)
             kcl.kcl_count(v, k, o)
             ws, ar = kcl.kcl_scratch_bytes(v)
             out["scratch_bytes"]["k=%d %s" % (k, o)] = {"workspace": ws, "arena": ar}
             v.free()
-    kcl.kcl_set_options(g, 0)
-    kcl.kcl_set_tuning(g, {})
+    g.free()
+    g = kcl.kcl_load_csr(*kclgen.rmat20(seed=1, scale=PRUNE_SCALE))
+    kcl.kcl_enable_timing(g, True)
+    out["calls"]["k=%d color (R-MAT scale %d)" % (PRUNE_K, PRUNE_SCALE)] = ablation_row(
+        g, PRUNE_K, "color", [("all on", 0, None), ("no colour prune", kcl.KCL_OPT_NO_COLOR_PRUNE, None)], args.steps)
     g.free()
     return out
 
