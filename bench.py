@@ -417,7 +417,10 @@ def roofline(per_call, steps, peaks, sm_mhz, modes=("count", "list")):
     (tests/golden/rmat20_work.json, split by out-degree) / that launch's
     CUDA-event time.  The units are the paper's: the id-ordered kernels close
     the same cliques with fewer words (compacted candidate sets) and fewer
-    rounds (shared chains), so a fraction may exceed 1."""
+    rounds (shared chains: one a clique, two when the root's id is its largest),
+    so a fraction may exceed 1 and says nothing about how busy the pipe is; for
+    listing `rounds_frac` is the fraction with the rounds that are executed for
+    the cliques kept, 1 + 1/k each on average."""
     work = _load_work()
     fam = {}
     for (k, o, m, c, ms, la, cl) in per_call:
@@ -447,10 +450,14 @@ def roofline(per_call, steps, peaks, sm_mhz, modes=("count", "list")):
     peak_g = sms * per_clk * sm_mhz * 1e6 / 1e9
     achieved = (wk / (avg_ms / 1e3) / 1e9) if wk else None
     kern = KERNEL_NAMES.get((o, m, ci), "listing launch of class %d" % ci)
+    rounds = None  # of the measured round rate, what the cliques' own rounds take
+    if achieved and m == "list":
+        rounds = achieved * (1 + 1 / k if kern.startswith("k_sub") else k) / (peak_g * k)
     tr = TRAFFIC.get((k, o, m, ci))
     return {"kernel": "%s (k=%d %s %s, roots with %d <= d+ <= %d)" % (kern, k, o, m, lo, hi),
             "bound": "alu", "achieved": achieved, "peak": peak_g, "unit": unit,
             "frac": (achieved / peak_g) if achieved else None,
+            "rounds_frac": rounds,
             "traffic": tr[0] if tr else None,
             "traffic_source": tr[1] if tr else None,
             "work_per_launch": wk, "roots": roots, "avg_ms": avg_ms,
