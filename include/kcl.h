@@ -300,7 +300,7 @@ kcl_status kcl_get_options(const kcl_graph *g, uint32_t *flags);
  * per-call workspace (one allocation of about 74 bytes per vertex and 2 per CSR
  * entry, grown to the largest graph seen) and the listing arena (shared-memory
  * spill of the largest subproblems, sized by k and the largest out-degree; the
- * few words a small graph needs lie in the workspace), in bytes.
+ * few words a small graph needs come out of the workspace), in bytes, each once.
  * The input CSR itself (8 (n+1) + 4 nnz bytes) is not included. */
 kcl_status kcl_scratch_bytes(const kcl_graph *g, uint64_t *workspace, uint64_t *arena);
 

@@ -1,4 +1,7 @@
-// BitCol on the GPU (Algorithm 6, Section VII).  For every root u of the
+// BitCol on the GPU (Algorithm 6, Section VII): the colour ordering's kernels for
+// k > 6, for root out-degrees above 1,024, and for any k without the colour prune
+// (the id-ordered kernels of kcl_sub.cu take the rest, so the unrolled forms for
+// k = 3..6 below serve those two cases only).  For every root u of the
 // degeneracy DAG with d+_u >= k-1 a group of threads (one warp for small
 // out-degrees, one CTA for large ones)
 //   1. builds G_u, the undirected subgraph induced by N+_u (Section VII-B), as

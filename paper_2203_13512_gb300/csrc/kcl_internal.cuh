@@ -102,7 +102,7 @@ struct Workspace {
     uint32_t *peel_deg = nullptr;    // n: degrees during the degeneracy peel
     uint32_t *frontier_a = nullptr;  // n
     uint32_t *frontier_b = nullptr;  // n
-    uint32_t *parent = nullptr;      // n: union-find forest (Pre-List)
+    uint32_t *parent = nullptr;      // n: smallest id of a vertex's closed neighbourhood (Pre-List)
     uint32_t *comp_n = nullptr;      // n: component sizes (by root)
     uint32_t *comp_flag = nullptr;   // n: 1 = clique component root
     uint32_t *outdeg = nullptr;      // n
@@ -121,7 +121,7 @@ struct Workspace {
     size_t arena_words = 0;
     DevResult *res = nullptr;
     DevResult *h_res = nullptr;      // pinned host mirror
-    PeelCtl *peel = nullptr;         // single-launch peel control block
+    PeelCtl *peel = nullptr;         // control block of the peel
     unsigned long long *vcount_pre = nullptr;  // batch: Pre-List counts by component root
     unsigned long long *vcks_pre = nullptr;    // batch: Pre-List checksums by component root
     const uint32_t *idmap = nullptr;           // batch: union vertex -> graph's own id
@@ -544,7 +544,6 @@ inline bool allow_max_smem(K kern) {
 
 // kcl_prep.cu
 int launch_validate(const kcl_graph *g, DevResult *res, cudaStream_t s);
-int launch_degrees(const kcl_graph *g, uint32_t *deg, cudaStream_t s);
 // Pre-Core (res zeroed first): the initial frontier and a few rounds; res->pre_nin
 // is the frontier that is left, 0 almost always.  launch_precore_rounds: more rounds.
 int launch_precore(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s);

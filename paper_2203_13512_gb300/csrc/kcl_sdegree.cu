@@ -1,4 +1,6 @@
-// SDegree on the GPU (Algorithm 5, Section VI): for every root u of the
+// SDegree on the GPU (Algorithm 5, Section VI): the degree ordering's kernels for
+// k > 6, for root out-degrees above 1,024, and for any k where lists are asked for
+// (the id-ordered kernels of kcl_sub.cu take the rest).  For every root u of the
 // degree-ordered DAG with d+_u >= k-1, one warp runs SDegreeList(k-1, {u},
 // N+_u) as an explicit-stack DFS over sorted candidate lists:
 //   for each v in C: skip v when d+_v <= l-2 (degree prune);
