@@ -21,8 +21,8 @@
 //     once per (node, a) and a clique costs one SplitMix64 round (two when
 //     the root's own id is the largest) instead of k and a merge.
 // Listing kernels of the 1M-vertex R-MAT graph (16 edges a vertex), before and
-// now: k = 5 colour count 179.3 -> 42.2 ms, k = 4 colour listing 201.2 -> 99.4
-// ms (2.06e10 records, 3.3 TB/s of stores; the stores alone would take 43 ms at
+// now: k = 5 colour count 179.3 -> 42.4 ms, k = 4 colour listing 201.2 -> 97.0
+// ms (2.06e10 records, 3.4 TB/s of stores; the stores alone would take 43 ms at
 // the 7.7 TB/s that a fill writes here, the hashes alone 83).  Counting is bound by the ALU pipe, listing by
 // issue slots around the hash round.  A kernel per k: with all of k = 3..6 in
 // one, 45.0 and 106.0 ms (registers, instruction cache).
