@@ -333,7 +333,7 @@ kcl_status kcl_scratch_bytes(const kcl_graph *g, uint64_t *workspace, uint64_t *
  *   another CTA and takes over some of its children when at least t =
  *   split[c] of them are left; 0 = off (default).
  * The id-ordered kernels (k <= 6, see the orderings above) use cta_warps only;
- * they share heavy roots between CTAs by a rule of their own.
+ * they share heavy roots between CTAs by a rule of their own (not when it is 1).
  * A graph starts with the defaults; views and batches start with the
  * defaults too. */
 typedef struct {
