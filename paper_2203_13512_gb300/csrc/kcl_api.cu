@@ -394,8 +394,9 @@ kcl_status run_front(kcl_graph *g, uint32_t k, kcl_ordering ord, const kcl_ring 
         if (w.h_res->pre_nin == 0) break;
         // more wide rounds than Pre-Core's launches: nothing has been counted,
         // listed or removed since (k_pl_check), so the rest follows once they are done
-        for (uint32_t nin = 1; nin;) {
-            T.add(0, launch_precore_rounds(g, kcore, w, 8, s));
+        uint32_t nin = w.h_res->pre_nin;
+        for (int rounds = 8; nin; rounds = std::min(2 * rounds, 128)) {
+            T.add(0, launch_precore_rounds(g, kcore, w, rounds, nin, s));
             KCL_TRY(read_u32(g, &w.res->pre_nin, &nin));
         }
         KCL_CK(cudaMemsetAsync(w.res, 0, sizeof(DevResult), s));

@@ -545,9 +545,10 @@ inline bool allow_max_smem(K kern) {
 // kcl_prep.cu
 int launch_validate(const kcl_graph *g, DevResult *res, cudaStream_t s);
 // Pre-Core (res zeroed first): the initial frontier and a few rounds; res->pre_nin
-// is the frontier that is left, 0 almost always.  launch_precore_rounds: more rounds.
+// is the frontier that is left, 0 almost always.  launch_precore_rounds: more rounds,
+// with blocks for frontiers of about `rows` vertices.
 int launch_precore(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s);
-int launch_precore_rounds(const kcl_graph *g, uint32_t k, Workspace &w, int rounds, cudaStream_t s);
+int launch_precore_rounds(const kcl_graph *g, uint32_t k, Workspace &w, int rounds, uint32_t rows, cudaStream_t s);
 int launch_prelist(const kcl_graph *g, uint32_t k, Workspace &w, int listing, cudaStream_t s);
 int launch_prelist_emit(const kcl_graph *g, uint32_t k, Workspace &w, uint32_t n_comps,
                         const kcl_ring *ring, cudaStream_t s);

@@ -143,9 +143,11 @@ __device__ __forceinline__ uint32_t warp_append(unsigned m, unsigned *count) {
 // graph took as long as that call (2.2 s), and takes 4.2 ms this way.  Short rounds
 // would cost a launch each; instead a launch's last block to finish runs the rounds
 // that follow while they have at most kPreTail vertices, and leaves wider ones to
-// the next launch (k = 5 count of a 2,000-vertex graph: 214 -> 206 us).
-constexpr uint32_t kPreTail = 2048;
-constexpr int kPreThreads = 512;
+// the next launch (k = 5 count of a 2,000-vertex graph: 214 -> 206 us; 100,000
+// rounds along a path 202 -> 60 ms; 200 rounds of 1,600 vertices 1.9 ms as launches,
+// 6.2 when the last block took up to 2,048, 1.8 in the cooperative launch).
+constexpr uint32_t kPreTail = 512;
+constexpr int kPreThreads = 1024;
 
 __global__ void k_precore_init(uint32_t n, const uint64_t *__restrict__ rp, uint32_t thr,
                                const uint8_t *__restrict__ kmap, uint8_t *alive, uint32_t *cdeg,
@@ -180,28 +182,37 @@ struct PreArgs {
     DevResult *res;
 };
 
-// One entry a lane (`in`: it has one): the neighbour loses a degree and may leave.
-__device__ __forceinline__ void precore_entry(const PreArgs &a, uint64_t x, bool in, uint32_t at, unsigned *next) {
-    uint32_t w = 0;
-    bool out = false;
-    if (in) {
-        w = a.col[x];
-        const uint32_t t = a.kmap ? a.kmap[w] - 1u : a.thr;
-        out = t > 0 && atomicSub(&a.cdeg[w], 1u) == t;  // fell from k-1 to k-2
+// Z entries a lane (x, x + 32, ... below e): their vertices lose a degree and may
+// leave.
+template <int Z>
+__device__ __forceinline__ void precore_entries(const PreArgs &a, uint64_t x, uint64_t e, uint32_t at,
+                                                unsigned *next) {
+    uint32_t w[Z];
+    bool out[Z];
+#pragma unroll
+    for (int z = 0; z < Z; z++) w[z] = x + 32 * z < e ? a.col[x + 32 * z] : 0xFFFFFFFFu;
+#pragma unroll
+    for (int z = 0; z < Z; z++) {
+        const uint32_t t = w[z] == 0xFFFFFFFFu ? 0u : a.kmap ? a.kmap[w[z]] - 1u : a.thr;
+        out[z] = t > 0 && atomicSub(&a.cdeg[w[z]], 1u) == t;  // fell from k-1 to k-2
     }
-    const unsigned m = __ballot_sync(0xffffffffu, out);
-    if (m) {
-        const uint32_t i = warp_append(m, next);
-        if (out) {
-            a.alive[w] = 0;
-            a.list[at + i] = w;
+#pragma unroll
+    for (int z = 0; z < Z; z++) {
+        const unsigned m = __ballot_sync(0xffffffffu, out[z]);
+        if (m) {
+            const uint32_t i = warp_append(m, next);
+            if (out[z]) {
+                a.alive[w[z]] = 0;
+                a.list[at + i] = w[z];
+            }
         }
     }
 }
 
 // The round of list[lo, lo + nin) by W warps, this one being number gw; the next
 // round is appended behind it.  Most rows are shorter than k: 8 lanes a row, and
-// the warp together for rows beyond 64 entries.
+// the warp together, four entries a lane, for rows beyond 64 entries (a hub's
+// 1M entries 17 -> 13 ms).
 __device__ void precore_round(const PreArgs &a, uint32_t lo, uint32_t nin, unsigned *next, uint32_t gw, uint32_t W) {
     const unsigned lane = lane_id();
     const uint32_t at = lo + nin;
@@ -216,16 +227,16 @@ __device__ void precore_round(const PreArgs &a, uint32_t lo, uint32_t nin, unsig
         const bool big = e - b > 64;
         const uint32_t most = __reduce_max_sync(0xffffffffu, big ? 0u : (uint32_t)(e - b));
         for (uint32_t x = lane & 7u; x - (lane & 7u) < most; x += 8)
-            precore_entry(a, b + x, !big && b + x < e, at, next);
+            precore_entries<1>(a, b + x, big ? 0ull : e, at, next);
         for (unsigned todo = __ballot_sync(0xffffffffu, big && (lane & 7u) == 0); todo; todo &= todo - 1) {
             const int j = __ffs(todo) - 1;
             const uint64_t rb = __shfl_sync(0xffffffffu, b, j), re = __shfl_sync(0xffffffffu, e, j);
-            for (uint64_t x = rb; x < re; x += 32) precore_entry(a, x + lane, x + lane < re, at, next);
+            for (uint64_t x = rb; x < re; x += 128) precore_entries<4>(a, x + lane, re, at, next);
         }
     }
 }
 
-__global__ void __launch_bounds__(kPreThreads) k_precore_round(const PreArgs a) {
+__global__ void __launch_bounds__(kPreThreads, 2) k_precore_round(const PreArgs a) {
     __shared__ unsigned next_s, last_s;
     // changed only by the last block, when every block has read them
     uint32_t lo = *(volatile unsigned *)&a.res->pre_lo, nin = *(volatile unsigned *)&a.res->pre_nin;
@@ -1238,9 +1249,9 @@ static PreArgs precore_args(const kcl_graph *g, uint32_t k, Workspace &w) {
     return PreArgs{g->rp, g->col, k - 1, k > 1 ? w.kmap : nullptr, w.alive, w.cdeg, w.members, w.res};
 }
 
-int launch_precore_rounds(const kcl_graph *g, uint32_t k, Workspace &w, int rounds, cudaStream_t s) {
+int launch_precore_rounds(const kcl_graph *g, uint32_t k, Workspace &w, int rounds, uint32_t rows, cudaStream_t s) {
     const PreArgs a = precore_args(g, k, w);
-    const int grid = grid_for((uint64_t)g->n * 8, kPreThreads, g->num_sms, 4);  // 8 lanes a row
+    const int grid = grid_for((uint64_t)rows * 8, kPreThreads, g->num_sms, 2);  // 8 lanes a row
     for (int i = 0; i < rounds; i++) k_precore_round<<<grid, kPreThreads, 0, s>>>(a);
     return rounds;
 }
@@ -1249,9 +1260,9 @@ int launch_precore(const kcl_graph *g, uint32_t k, Workspace &w, cudaStream_t s)
     const PreArgs a = precore_args(g, k, w);
     k_precore_init<<<grid_for(g->n, kBlock, g->num_sms), kBlock, 0, s>>>(g->n, a.rp, a.thr, a.kmap, a.alive, a.cdeg,
                                                                         a.list, a.res);
-    // wide rounds by size: 400,000 vertices at k = 10 have three of more than
-    // kPreTail vertices, R-MAT graphs up to 2^20 vertices one
-    return 1 + launch_precore_rounds(g, k, w, g->n <= kPreTail ? 1 : g->n <= (1u << 16) ? 2 : 3, s);
+    // wide rounds by size: 400,000 vertices at k = 10 have four of more than
+    // kPreTail vertices, R-MAT graphs up to 2^20 vertices one or two
+    return 1 + launch_precore_rounds(g, k, w, g->n <= 2048 ? 1 : g->n <= (1u << 16) ? 2 : 4, g->n, s);
 }
 
 int launch_prelist(const kcl_graph *g, uint32_t k, Workspace &w, int listing, cudaStream_t s) {

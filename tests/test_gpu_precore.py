@@ -31,8 +31,8 @@ def _unravelling(width, layers):
     return kclgen.from_edges(n + 67, np.concatenate([e, pairs[pairs[:, 0] < pairs[:, 1]]]))
 
 
-# 2 * width below and above the width that a launch's last block takes on; up to
-# 2, 3 and then 8 launches at a time
+# 2 * width below and above the width that a launch's last block takes on; rounds that
+# fit the first launches, one more group of them and several
 @pytest.mark.parametrize("width,layers", [(20, 11), (900, 40), (1500, 20), (1500, 60), (5000, 12)])
 def test_many_wide_rounds(width, layers):
     import paper_2203_13512_gb300 as kcl
